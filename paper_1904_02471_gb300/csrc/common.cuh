@@ -20,7 +20,7 @@ namespace lbm {
 
 constexpr int NOBS = 4;  // sum rho (minus the storage offset), sum j_x, sum j_y, probe sum
 
-struct LatDesc {
+struct alignas(16) LatDesc {   // copied in 16-byte chunks
     void* buf[3];           // CS: buf[0]/buf[1] ping-pong; FD: f^n, f^(1), f^(2)
     int nx, ny;
     int pitch;              // row pitch in elements (multiple of 32)

@@ -142,10 +142,13 @@ void Engine::invalidate_graph() {
     graph_chunk_ = 0;
 }
 
-// Default grid of a group: one block per work item (tile) when the lattices
-// are fixed (the hardware scheduler balances the tiles; the tuner picked this
-// for every workload measured, e.g. CS D2Q9 8192^2 in place 90 GLUPS against
-// 72 with one block set per SM), one block set per SM for a server's engine,
+// Default grid of a group. Fixed lattices: CS and the temporally blocked FD
+// step, one block per work item (tile; the hardware scheduler balances the
+// tiles; the tuner picked this for every workload measured, e.g. CS D2Q9 8192^2
+// in place 90 GLUPS against 72 with one block set per SM); FD stages, one block
+// per SM (a block prepares its next tile while it works on one: 1.06 ms per
+// stage of FD 16-velocity 4096^2 against 1.7 ms with one block per tile). One
+// block set per SM for a server's engine,
 // whose lattices change under a captured graph (the blocks then loop over
 // the items), or grid_mult_ block sets, so that each block covers fewer items
 // and retires sooner (SMs then free up for another stream's kernels).
@@ -156,8 +159,36 @@ int Engine::persistent_grid(const Group& g, int tile) const {
 }
 
 int Engine::default_grid(const Group& g, int tile) const {
-    if (!dynamic_ && g.total_items > 0) return g.total_items;
+    if (!dynamic_ && g.total_items > 0)
+        return g.model == LBM_FD && g.scheme != LBM_TS_RK3_FUSED ? std::min(g.total_items, persistent_grid(g, tile))
+                                                                 : g.total_items;
     return persistent_grid(g, tile) * std::max(1, grid_mult_);
+}
+
+// Default tile of an FD group of fixed lattices: the variant with the least
+// rounds x (rows + c), rounds = tiles per SM rounded up, c the cost of a tile
+// beside its rows (halo, moments, first faces, block start) in rows. Measured
+// per tile and stage, 16 velocities: FP32 4.96 / 2.92 / 2.17 / 1.95 us and FP64
+// 204 / 110 / 64 / 40 us with 16 / 8 / 4 / 2 rows: c = 6.4 and 1.4. Small
+// lattices get small tiles (more SMs at work: FP64 60^2, 122 us per step with
+// 2 rows, 331 with 8), large ones tall tiles (FP32 2048^2, 0.80 ms per step
+// with 16 rows, 0.95 with 8).
+int Engine::default_fd_tile(const Group& g) const {
+    const double c = g.precision == LBM_FP64 ? 1.4 : 6.4;
+    int best = g.tile;
+    double best_cost = 1e300;
+    for (int t = 0; t < (int)FD_NTILES; ++t) {
+        if (!fd_variant_fits(g.precision, g.q1, t, g.scheme)) continue;
+        const int tx = fd_tile_tx(t), ty = fd_tile_ty(t);
+        long long items = 0;
+        for (int li : g.members) items += (long long)((lat[li].spec.nx + tx - 1) / tx) * ((lat[li].spec.ny + ty - 1) / ty);
+        const double cost = (double)((items + sm_count_ - 1) / sm_count_) * (ty + c);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = t;
+        }
+    }
+    return best;
 }
 
 int Engine::open(void* stream) {
@@ -248,6 +279,7 @@ int Engine::add_lattice(const lbm_spec* spec, int* index, bool upload) {
         g.precision = s.precision;
         g.scheme = s.scheme;
         g.tile = s.model == LBM_CS ? (int)CS_B256x32 : (int)FD_T32x8;
+        if (s.model == LBM_FD && s.scheme != LBM_TS_RK3_FUSED && (long long)s.nx * s.ny >= 1 << 20) g.tile = (int)FD_T32x16;
         // the fused FD kernel's largest tiles do not fit every set and precision
         if (s.model == LBM_FD && s.scheme == LBM_TS_RK3_FUSED && !fd_variant_fits(s.precision, s.q_per_axis, g.tile, s.scheme))
             g.tile = FD_T32x4;
@@ -294,6 +326,8 @@ int Engine::create(const lbm_spec* specs, int n, void* stream) {
         rc = add_lattice(&specs[i], nullptr, false);
         if (rc) return rc;
     }
+    for (auto& g : groups)
+        if (g.model == LBM_FD) g.tile = default_fd_tile(g);
     return upload_all();
 }
 

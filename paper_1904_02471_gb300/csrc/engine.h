@@ -162,6 +162,7 @@ class Engine {
     int sm_count() const { return sm_count_; }
     int default_grid(const Group& g, int tile) const;
     int persistent_grid(const Group& g, int tile) const;
+    int default_fd_tile(const Group& g) const;
     int tune(int trial_steps, std::string* report);
 
     int chunk = 32;          // steps per captured graph

@@ -7,17 +7,17 @@
 // One launch = one stage for every lattice of the group. The moments (rho, u)
 // and so f^eq are taken from that stage's input, as the BGK term belongs to L.
 //
-// Per tile (TX x TY nodes):
-//   1. every population plane of the stage input is staged in shared memory
-//      with a periodic halo of 3 nodes (the WENO-5 stencil reach); the
-//      moments come from there,
-//   then per group of G populations:
-//   2. per group of G populations, every interface value is computed once
-//      and stored: (TX+1) x TY faces normal to x and TX x (TY+1) normal to y
-//      (a face is shared by the two nodes it separates, which also makes the
-//      flux form conservative),
-//   3. after one barrier each node takes its flux differences, adds the BGK
-//      term and combines with f^n for the stage.
+// Per tile (TX x TY nodes), two kinds of warps of a block:
+//   preparing warps, one tile ahead of the others: copy every population of
+//   the stage input with a periodic halo of 3 nodes (the WENO-5 stencil reach)
+//   to shared memory and form the moments of the tile's nodes,
+//   march warps: each takes one population up the rows of the tile. Along y
+//   the stencil slides in registers (an interface value is computed once, as
+//   the face above a row and then the face below the next); along x a lane
+//   computes the faces on the upwind side of its nodes and takes the others
+//   from the neighbouring lane. Both sides of an interface use the same value,
+//   so the flux form is conservative. The node then adds the BGK term and
+//   combines with f^n for the stage.
 // The WENO-5 face value is upwinded by the sign of the (constant) velocity
 // component: for v > 0 the face i+1/2 is reconstructed from f_{i-2..i+2},
 // for v < 0 from f_{i+3..i-1} (mirror image). Components equal to 0 (the
@@ -28,6 +28,8 @@
 // buf[2] = f^(2). Storage offset as in the CS kernel (deviation form for
 // FP32, full f for FP64): WENO differences and the stage combination are
 // unchanged by the constant offset w_k rho0.
+#include <atomic>
+
 #include "fd_common.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
@@ -35,144 +37,280 @@
 namespace lbm {
 
 // Column sums cs[ix] = sum_iy g(ix + Q1 iy) and row sums rs[iy] =
-// sum_ix g(ix + Q1 iy) of a quantity over the product set.
+// sum_ix g(ix + Q1 iy) of a quantity over the product set, then its zeroth
+// and first moments sum g, sum g v_x, sum g v_y (v_x depends on ix only, v_y
+// on iy only): fewer operations than K products per component.
 template <typename T, int Q1, typename Fn>
-__device__ __forceinline__ void sum_cols_rows(Fn g, T (&cs)[Q1], T (&rs)[Q1]) {
+__device__ __forceinline__ void set_moments(Fn g, typename Lanes<T>::V& m0, typename Lanes<T>::V& mx,
+                                            typename Lanes<T>::V& my) {
+    using P = Lanes<T>;
+    using V = typename P::V;
+    V cs[Q1], rs[Q1];
 #pragma unroll
     for (int iy = 0; iy < Q1; ++iy)
 #pragma unroll
         for (int ix = 0; ix < Q1; ++ix) {
-            const T v = g(ix + Q1 * iy);
-            cs[ix] = iy == 0 ? v : cs[ix] + v;
-            rs[iy] = ix == 0 ? v : rs[iy] + v;
+            const V v = g(ix + Q1 * iy);
+            cs[ix] = iy == 0 ? v : P::add(cs[ix], v);
+            rs[iy] = ix == 0 ? v : P::add(rs[iy], v);
         }
-}
-// Zeroth and first moments from column and row sums: sum g, sum g v_x,
-// sum g v_y (v_x depends on ix only, v_y on iy only).
-template <typename T, int Q1>
-__device__ __forceinline__ void moments_of_sums(const T (&cs)[Q1], const T (&rs)[Q1], T& m0, T& mx, T& my) {
     m0 = cs[0];
 #pragma unroll
-    for (int i = 1; i < Q1; ++i) m0 += cs[i];
-    mx = T(0);
-    my = T(0);
+    for (int i = 1; i < Q1; ++i) m0 = P::add(m0, cs[i]);
+    mx = P::mulc(cs[0], (T)GH<Q1>::v(0));
+    my = P::mulc(rs[0], (T)GH<Q1>::v(0));
 #pragma unroll
-    for (int i = 0; i < Q1; ++i) {
+    for (int i = 1; i < Q1; ++i) {
         if (GH<Q1>::v(i) != 0.0) {
-            mx += (T)GH<Q1>::v(i) * cs[i];
-            my += (T)GH<Q1>::v(i) * rs[i];
+            mx = P::fmac(cs[i], (T)GH<Q1>::v(i), mx);
+            my = P::fmac(rs[i], (T)GH<Q1>::v(i), my);
         }
     }
 }
-// v_k . u and v_k . j + d of population k from per-axis products: the 1D set
-// is symmetric (v_{Q1-1-i} = -v_i), so v_i u_x and v_i j_x are formed for
-// the upper half of the nodes and negated for the lower half; v_iy u_y and
-// v_iy j_y + d once per row (shared by the Q1 populations of the row).
-template <typename T, int Q1>
-struct EqTerms {
-    T ux, uy, jx, jy, d;
-    __device__ __forceinline__ T xu(int ix) const {
-        return GH<Q1>::v(ix) == 0.0 ? T(0)
-               : (2 * ix >= Q1 ? (T)GH<Q1>::v(ix) * ux : -((T)GH<Q1>::v(Q1 - 1 - ix) * ux));
+
+// The equilibrium at a node as five numbers (px, py, jx, jy, e0):
+//   stored f^eq_k = w_k (q_k + v_k . j + e0), i.e. Eq. (herfeq) minus w_k rho0.
+// FP32: p = j / sqrt(2 rho), q_k = (v_k . p)^2 = rho/2 (v_k . u)^2, e0 = dr - p^2;
+// FP64: p = u/2, q_k = (v_k . p)(v_k . j), e0 = dr - j . p (a square root
+// would cost more on the FP64 pipe than it saves).
+template <typename T>
+struct Equil {
+    using P = Lanes<T>;
+    using V = typename P::V;
+    V px, py, jx, jy, e0;
+    __device__ __forceinline__ void set(V rho, V dr, V jx_, V jy_) {
+        jx = jx_;
+        jy = jy_;
+        if constexpr (sizeof(T) == 4) {
+            const V s = P::rsqrt(P::add(rho, rho));
+            px = P::mul(jx, s);
+            py = P::mul(jy, s);
+            e0 = P::fma(P::neg(py), py, P::fma(P::neg(px), px, dr));
+        } else {
+            const V h = P::mulc(P::rcp(rho), T(0.5));
+            px = P::mul(jx, h);
+            py = P::mul(jy, h);
+            e0 = P::fma(-jy, py, P::fma(-jx, px, dr));
+        }
     }
-    __device__ __forceinline__ T xj(int ix) const {
-        return GH<Q1>::v(ix) == 0.0 ? T(0)
-               : (2 * ix >= Q1 ? (T)GH<Q1>::v(ix) * jx : -((T)GH<Q1>::v(Q1 - 1 - ix) * jx));
-    }
-    __device__ __forceinline__ T xi(int k) const {
-        const int ix = k % Q1, iy = k / Q1;
-        if (GH<Q1>::v(iy) == 0.0) return xu(ix);
-        const T yv = (T)GH<Q1>::v(iy) * uy;
-        return GH<Q1>::v(ix) == 0.0 ? yv : xu(ix) + yv;
-    }
-    __device__ __forceinline__ T lin(int k) const {
-        const int ix = k % Q1, iy = k / Q1;
-        const T yl = GH<Q1>::v(iy) == 0.0 ? d : (T)GH<Q1>::v(iy) * jy + d;
-        return GH<Q1>::v(ix) == 0.0 ? yl : xj(ix) + yl;
+    // (f^eq_k) / w_k; vx, vy: the population's velocity, broadcast
+    __device__ __forceinline__ V over_w(V vx, V vy) const {
+        const V xi = P::fma(vx, px, P::mul(vy, py));
+        if constexpr (sizeof(T) == 4) {
+            return P::fma(xi, xi, P::fma(vx, jx, P::fma(vy, jy, e0)));
+        } else {
+            const V xj = P::fma(vx, jx, P::mul(vy, jy));
+            return P::add(P::fma(xi, xj, xj), e0);
+        }
     }
 };
 
-// Tile geometry: TX = 32 nodes along x (one warp per row), TY rows. The
-// staged halo tile of a population has HY = TY + 6 rows of HXP = 40 values,
-// columns x0 - 4 .. x0 + 35 (16-byte aligned rows; the stencil needs
-// x0 - 3 .. x0 + 34), rows y0 - 3 .. y0 + TY + 2.
+// The same for all populations of a set in turn (compile-time k), with the
+// terms in v_y formed once per row of the product set. The operations and
+// their order are Equil::over_w's: the residual moments below have to be those
+// of the equilibrium the update uses, to the last bit (with products and sums
+// rounded apart here, the FP32 decay rate of an IMEX run is off by 2.6e-4).
+template <typename T, int Q1>
+struct EquilAll {
+    using P = Lanes<T>;
+    using V = typename P::V;
+    V px, jx, yp[Q1], yj[Q1], e0;
+    __device__ __forceinline__ explicit EquilAll(const Equil<T>& e) : px(e.px), jx(e.jx), e0(e.e0) {
+#pragma unroll
+        for (int i = 0; i < Q1; ++i) {
+            const T v = (T)GH<Q1>::v(i);
+            yp[i] = P::mulc(e.py, v);
+            yj[i] = sizeof(T) == 4 ? P::fmac(e.jy, v, e.e0) : P::mulc(e.jy, v);
+        }
+    }
+    // f^eq_k / w_k
+    __device__ __forceinline__ V over_w(int k) const {
+        const int ix = k % Q1, iy = k / Q1;
+        const T v = (T)GH<Q1>::v(ix);
+        const V xi = P::fmac(px, v, yp[iy]), vj = P::fmac(jx, v, yj[iy]);
+        if constexpr (sizeof(T) == 4) return P::fma(xi, xi, vj);
+        else return P::add(P::fma(xi, vj, vj), e0);
+    }
+};
+
+// Velocity tables of a product set for run-time population indices; the
+// values are those the unrolled loops fold to immediates.
+template <typename T, int Q1>
+struct SetTable {
+    T vx[Q1 * Q1], vy[Q1 * Q1], w[Q1 * Q1];
+    constexpr SetTable() : vx{}, vy{}, w{} {
+        for (int k = 0; k < Q1 * Q1; ++k) {
+            vx[k] = (T)vx_of<Q1>(k);
+            vy[k] = (T)vy_of<Q1>(k);
+            w[k] = (T)w_of<Q1>(k);
+        }
+    }
+};
+template <typename T, int Q1>
+__constant__ SetTable<T, Q1> c_set{};
+
+// Geometry of a tile: TX = 32 nodes along x by TY rows. A lane holds N
+// neighbouring nodes of a row (Lanes<T>::V: a pair for FP32, so that every
+// packed FP32x2 instruction does the same arithmetic for two nodes; one for
+// FP64); a row takes LC = 32 / N lanes and the N row groups of a warp lie H =
+// TY / N rows apart. A population's staged tile has RT = TY + 6 rows of HXP =
+// 40 columns, x0 - 4 .. x0 + 35 (16-byte aligned; the stencils need x0 - 3 ..
+// x0 + 34). Rows are marched in the direction of v_y by a run-time row stride,
+// so the code differs only by the sign of v_x and stays in the instruction
+// cache.
 constexpr int FD_TX = 32;
 constexpr int FD_HXP = 40;
 
-// Populations whose faces are evaluated between two barriers (a group): 4,
-// or 2 where four face groups would not fit next to the halo tiles (FP64, 25
-// velocities), or 8 for FP32 32 x 8 tiles: warp p evaluates the edge faces of
-// the group's p-th population, so a group of as many populations as the tile
-// has warps gives every warp the same work between two barriers.
-template <typename T, int Q1, int TY>
-__host__ __device__ constexpr int fd_group() {
-    return (sizeof(T) == 8 && Q1 == 5) ? 2 : (sizeof(T) == 4 && TY == 8 ? 8 : 4);
-}
-// Face buffers: two alternate between groups (one barrier per group); a
-// group of 8 has one (two barriers per group, the same shared memory).
-template <typename T, int Q1, int TY>
-__host__ __device__ constexpr int fd_face_bufs() { return fd_group<T, Q1, TY>() == 8 ? 1 : 2; }
+template <typename T, int Q1, int TY, bool IMEX>
+struct FdGeo {
+    static constexpr int N = Lanes<T>::N;
+    static constexpr int K = Q1 * Q1;
+    static constexpr int H = TY / N;
+    static constexpr int RT = TY + 6;
+    static constexpr int PL = RT * FD_HXP;
+    // A march is one population and S-th of the tile's rows (9 velocities:
+    // halves, for more warps). Warps per block: NM march warps, NA preparing.
+    static constexpr int S = Q1 == 3 && sizeof(T) == 4 && H >= 4 ? 2 : 1;
+    static constexpr int HS = H / S;
+    static constexpr int NM = Q1 == 5 ? 13 : K * S;
+    static constexpr int NA = Q1 == 4 ? (IMEX ? 8 : 4) : (Q1 == 3 && S == 2 ? 4 : 7);
+    static constexpr int NT = (NM + NA) * 32;
+    // registers per thread of the two kinds of warps (FP32, 16 velocities: the
+    // launch's registers are split between the warpgroups; 0: not split)
+    static constexpr bool SPLIT = Q1 == 4 && sizeof(T) == 4;
+    static constexpr int RM = SPLIT ? (IMEX ? 80 : 104) : 0, RA = SPLIT ? (IMEX ? 80 : 64) : 0;
+    static constexpr size_t n_mom = (size_t)5 * TY * FD_TX;
+    static constexpr size_t n_edge = ((size_t)K * TY + 3) / 4 * 4;
+    static constexpr size_t buf = (size_t)K * PL + n_mom + n_edge;   // values of a tile buffer
+    // two tile buffers (the next item is prepared while one is marched) where
+    // they fit the device's 227 KiB next to 3 KiB of static shared memory
+    static constexpr int NB = sizeof(T) * 2 * buf + sizeof(double) * NA * NOBS <= 224 * 1024 ? 2 : 1;
+    static constexpr size_t bytes = sizeof(T) * NB * buf + sizeof(double) * NA * NOBS;
+};
 
-template <typename T, int Q1, int TY>
-__host__ __device__ constexpr size_t fd_smem_bytes() {
-    return sizeof(T) * ((size_t)Q1 * Q1 * (TY + 6) * FD_HXP +
-                        fd_face_bufs<T, Q1, TY>() * fd_group<T, Q1, TY>() * ((FD_TX + 1) * TY + FD_TX * (TY + 1))) +
-           sizeof(double) * (FD_TX * TY / 32) * NOBS;
+// N neighbouring values from shared or global memory (aligned to the pair).
+__device__ __forceinline__ float2 ldv(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ double ldv(const double* p) { return *p; }
+__device__ __forceinline__ void stv(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
+__device__ __forceinline__ void stv(double* p, double v) { *p = v; }
+__device__ __forceinline__ void ldv2(const float* p, float2& a, float2& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ldv2(const double* p, double& a, double& b) {
+    const double2 v = *reinterpret_cast<const double2*>(p);
+    a = v.x;
+    b = v.y;
+}
+__device__ __forceinline__ void stv2(float* p, float2 a, float2 b) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void stv2(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
+// Read again instead of kept in registers since the last read.
+__device__ __forceinline__ float2 ldv_again(const float* p) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(smem_addr(p)));
+    return v;
+}
+__device__ __forceinline__ double ldv_again(const double* p) { return *p; }
+// The same through global addresses (the state pointers come from memory, so
+// the compiler takes them for generic ones).
+__device__ __forceinline__ float2 ldg_v(const float* p) {
+    float2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ double ldg_v(const double* p) {
+    double v;
+    asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ void stg_v(float* p, float2 v) {
+    asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void stg_v(double* p, double v) {
+    asm volatile("st.global.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void stg_1(float* p, float v) {
+    asm volatile("st.global.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void stg_1(double* p, double v) { stg_v(p, v); }
+
+// The node differences d1 .. d4 (weno5_diff) of the x-face on the upwind side
+// of a lane's nodes, from row pointer t (column -4 of the lane's first node);
+// SX: sign of v_x. Returns the nodes' own values.
+template <int SX>
+__device__ __forceinline__ float2 x_diffs(const float* t, float2& d1, float2& d2, float2& d3, float2& d4) {
+    const float2 B = ldv(t + 2), C = ldv(t + 4), E = ldv(t + 6);
+    if constexpr (SX > 0) {
+        const float2 A = ldv(t);
+        d1 = make_float2(A.y - B.x, B.x - B.y);
+        d2 = make_float2(B.x - B.y, B.y - C.x);
+        d3 = make_float2(B.y - C.x, C.x - C.y);
+        d4 = make_float2(C.x - C.y, C.y - E.x);
+    } else {
+        const float2 G = ldv(t + 8);
+        d1 = make_float2(E.y - E.x, G.x - E.y);
+        d2 = make_float2(E.x - C.y, E.y - E.x);
+        d3 = make_float2(C.y - C.x, E.x - C.y);
+        d4 = make_float2(C.x - B.y, C.y - C.x);
+    }
+    return C;
+}
+template <int SX>
+__device__ __forceinline__ double x_diffs(const double* t, double& d1, double& d2, double& d3, double& d4) {
+    const double a = t[4 - 3 * SX], b = t[4 - 2 * SX], c = t[4 - SX], d = t[4], e = t[4 + SX];
+    d1 = a - b;
+    d2 = b - c;
+    d3 = c - d;
+    d4 = d - e;
+    return d;
+}
+// The faces on the downwind side of a lane's nodes: those on the upwind side
+// of the next nodes in the direction of v_x, the outermost lane's from `edge`.
+template <int SX>
+__device__ __forceinline__ float2 x_next(float2 f, float edge, bool outer) {
+    if constexpr (SX > 0) {
+        const float n = __shfl_down_sync(0xffffffffu, f.x, 1);
+        return make_float2(f.y, outer ? edge : n);
+    } else {
+        const float n = __shfl_up_sync(0xffffffffu, f.y, 1);
+        return make_float2(outer ? edge : n, f.x);
+    }
+}
+template <int SX>
+__device__ __forceinline__ double x_next(double f, double edge, bool outer) {
+    const double n = SX > 0 ? __shfl_down_sync(0xffffffffu, f, 1) : __shfl_up_sync(0xffffffffu, f, 1);
+    return outer ? edge : n;
 }
 
-// Resident blocks per SM the register allocation is bounded for: 1024
-// threads per SM for FP32, i.e. at most 64 registers per thread (shared
-// memory, 53.5 KiB per 256-thread block for 16 populations, allows as many:
-// four blocks in 228 KiB); 512 threads (128 registers) for FP64.
-// The IMEX stage kernels hold more values per thread (the stage input and P
-// at the node): their FP32 variants are bounded for 512 threads per SM (128
-// registers) instead.
-template <typename T, int TY, bool IMEX = false>
-constexpr int fd_min_blocks() {
-    return ((sizeof(T) == 4 ? (IMEX ? 512 : 1024) : 512) / (FD_TX * TY)) > 0
-               ? (sizeof(T) == 4 ? (IMEX ? 512 : 1024) : 512) / (FD_TX * TY)
-               : 1;
-}
+template <int S>
+struct Const {
+    static constexpr int value = S;
+};
 
 // IMEX-SSP2(2,2,2) (LBM_TS_IMEX): gamma of the implicit tableau, 1 - 1/sqrt 2.
 constexpr double IMEX_GAMMA = 0.29289321881345247560;
 
-// IMEX: the implicit BGK part of a stage in closed form, at every staged node
-// of the tile. The stage value Y solves Y = u + dt g C(Y), C(Y) = -(Y -
-// f^eq(Y)) / tau; the collision conserves rho and rho u (Eq. herfeq has the
-// moments of Eq. f_moments_discrete), so Y has the moments of u, f^eq(Y) =
-// f^eq(u), and Y = (u + lam f^eq(u)) / (1 + lam), lam = g dt / tau. Values
-// in the storage form (deviations from w_k rho0 for FP32, r0 = rho0; full f
-// for FP64, r0 = 0): the map is linear, the offsets carry over.
-template <typename T, int Q1>
-__device__ __forceinline__ void imex_stage_values(T* tiles, int hxy, T r0, T lam, T il, int tid, int nt) {
-    constexpr int K = Q1 * Q1;
-    for (int pos = tid; pos < hxy; pos += nt) {
-        T dr = T(0), jx = T(0), jy = T(0);
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const T u = tiles[k * hxy + pos];
-            dr += u;
-            if (vx_of<Q1>(k) != 0.0) jx += u * (T)vx_of<Q1>(k);
-            if (vy_of<Q1>(k) != 0.0) jy += u * (T)vy_of<Q1>(k);
-        }
-        const T rho = r0 + dr;
-        const T inv = T(1) / rho;
-        const T ux = jx * inv, uy = jy * inv;
-        const T usq = ux * ux + uy * uy, hr = T(0.5) * rho;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const T vx = (T)vx_of<Q1>(k), vy = (T)vy_of<Q1>(k);
-            const T xi = vx * ux + vy * uy;
-            const T geq = (T)w_of<Q1>(k) * (hr * (xi * xi - usq) + (vx * jx + (vy * jy + dr)));
-            tiles[k * hxy + pos] = (tiles[k * hxy + pos] + lam * geq) * il;
-        }
-    }
-}
-
+// What bounds it. FP32: the register file and the FP32 pipe. A packed FP32x2
+// multiply-add with three distinct operand pairs issues every 3.2 cycles, with
+// two every 2.2 (measured), so operands count as much as operations: literals
+// go into scalar instructions as immediates, products that share a term are
+// folded. FP64: the FP64 pipe (1/64 of the FP32 rate).
+// Why this split. With every warp doing all parts of a tile in turn, copies,
+// barriers and the moments left the pipe idle for half of the time (1.19 ms
+// per stage of FD 16-velocity 4096^2 FP32 however the tile was cut). Here the
+// preparing warps' work overlaps the march, which never waits for memory: f^n
+// is loaded a march ahead, the rest is in shared memory. Stages of that lattice:
+// 1.19 / 1.13 / 1.13 -> 0.96 / 1.00 / 1.03 ms; FP64 256^2: 275 -> 200 us (fewer
+// operations per face and node, one reciprocal instead of a division).
+// Named barriers hand the buffers over: waiting warps take no issue slots
+// (polling an mbarrier took 10% of them).
+//
 // One stage of the FD update. IMEX = false: SSP-RK3 stage `stage` (1..3).
 // IMEX = true: stage 1 or 2 of IMEX-SSP2(2,2,2) with explicit WENO-5
-// advection A and implicit BGK C. With Y_i the stage values (above), the
+// advection A and implicit BGK C. With Y_i the stage values (below), the
 // scheme's
 //   Y_2 = f^n + dt A(Y_1) + (1 - 2g) dt C(Y_1) + g dt C(Y_2),
 //   f^{n+1} = f^n + dt/2 (A(Y_1) + A(Y_2) + C(Y_1) + C(Y_2))
@@ -185,451 +323,476 @@ __device__ __forceinline__ void imex_stage_values(T* tiles, int hxy, T r0, T lam
 // input (f^n or Z): no difference of nearly equal values is multiplied by
 // dt/tau, so the rounding stays small however stiff the collision is.
 template <typename T, int Q1, int TY, bool IMEX>
-__global__ void __launch_bounds__(FD_TX* TY, (fd_min_blocks<T, TY, IMEX>())) fd_stage_kernel(GroupDev g, int j, int stage) {
-    using P = Pr<T>;
+__global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel(GroupDev g, int j, int stage) {
+    using Ge = FdGeo<T, Q1, TY, IMEX>;
+    using P = Lanes<T>;
     using V = typename P::V;
-    constexpr int K = Q1 * Q1;
-    constexpr int TX = FD_TX, HXP = FD_HXP;
-    constexpr int NT = TX * TY;
-    constexpr int HY = TY + 6, HXY = HY * HXP;
-    constexpr int NFX = (TX + 1) * TY;   // faces normal to x: [TY][TX + 1]
-    constexpr int NFY = TX * (TY + 1);   // faces normal to y: [TY + 1][TX]
-    constexpr int NF = NFX + NFY;
-    constexpr int VEC = 16 / sizeof(T);   // values per 16-byte copy
-    constexpr int RV = HXP / VEC;         // 16-byte chunks per staged row
+    constexpr int K = Ge::K, N = Ge::N, H = Ge::H, RT = Ge::RT, PL = Ge::PL, NM = Ge::NM, NA = Ge::NA, NB = Ge::NB, S = Ge::S,
+                  HS = Ge::HS;
+    constexpr int TX = FD_TX, HXP = FD_HXP, LC = TX / N;
+    constexpr int VEC = 16 / (int)sizeof(T);   // values per 16-byte copy
+    constexpr int CH = HXP / VEC;              // 16-byte chunks per staged row
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int G = fd_group<T, Q1, TY>();
-    constexpr int FB = fd_face_bufs<T, Q1, TY>();
-    // 16-velocity set: populations 2q and 2q+1 (nodes ix = 0, 1 or 2, 3 of
-    // one row of the product set) have the same signs of both velocity
-    // components, so the same upwind stencils: their faces are evaluated and
-    // stored side by side
-    constexpr bool PAIRS = Q1 == 4;
-    static_assert(!PAIRS || (GH<4>::v(0) < 0 && GH<4>::v(1) < 0 && GH<4>::v(2) > 0 && GH<4>::v(3) > 0 && G % 2 == 0),
-                  "pairs (2q, 2q+1) must share their upwind directions");
-    T* tiles = reinterpret_cast<T*>(smem_raw);          // [K][HY][HXP]
-    T* faces = tiles + (size_t)K * HXY;                  // [FB][G][NF]
-    double* red = reinterpret_cast<double*>(faces + FB * G * NF);
-    __shared__ long long s_row[HY];                      // wrapped row offsets (edge tiles)
-    __shared__ int s_col[HXP];                           // wrapped columns (edge tiles)
-    __shared__ int s_obs;                                // record observables for this item
+    // NB tile buffers: [K][RT][HXP] staged values; per node the corrected
+    // moments, [TY][TX / N][2] (px, py), the same (jx, jy), [TY][TX] e0; [K][TY]
+    // faces beyond the outermost lane. Named barriers hand them over (2, 3:
+    // prepared; 4, 5: marched)
+    T* bufs = reinterpret_cast<T*>(smem_raw);
+    double* red = reinterpret_cast<double*>(bufs + NB * Ge::buf);
+    // the lattices' first items and whether they sit this step out (up to
+    // LATS of them; more are looked up in global memory), and the block's items
+    // in turn with their lattices' descriptors and tile origins
+    constexpr int LATS = 256;
+    __shared__ int s_begin[LATS];
+    __shared__ unsigned char s_dead[LATS];
+    __shared__ __align__(16) LatDesc s_desc[4];
+    __shared__ int s_item[4];
 
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int grp = lane / LC, c0 = (lane % LC) * N;   // row group and first column of the lane's nodes
+    constexpr int DCH = sizeof(LatDesc) / 16;          // 16-byte chunks of a descriptor
+    static_assert(sizeof(LatDesc) % 16 == 0 && DCH <= 32, "descriptors are copied in 16-byte chunks by one warp");
+    // a lone lattice's descriptor is read while the group's header is on its way
+    if (tid < DCH) reinterpret_cast<uint4*>(s_desc)[tid] = reinterpret_cast<const uint4*>(g.desc)[tid];
     const int n_lat = g.hdr[0];
     const int total = g.hdr[1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int tid = ty * TX + tx;
+    if (n_lat > 1 && n_lat <= LATS)
+        for (int i = tid; i < n_lat; i += Ge::NT) {
+            s_begin[i] = g.item_begin[i];
+            s_dead[i] = (long long)j >= g.desc[i].remaining;
+        }
+    __syncthreads();
     const int in_idx = IMEX ? (stage == 1 ? 0 : 1) : (stage == 1 ? 0 : (stage == 2 ? 1 : 2));
     const int out_idx = IMEX ? (stage == 1 ? 1 : 0) : (stage == 1 ? 1 : (stage == 2 ? 2 : 0));
     // the stage reads its input at its own node from global memory too (IMEX:
     // the staged tile holds the stage values Y instead), and f^n (RK3 stages 2, 3)
     const bool node_in = IMEX || stage != 1;
-    // stage weights: f^(s) = f^n + cb ((u - f^n) + dt L(u)), i.e. the Shu-Osher
-    // combinations 3/4 f^n + 1/4 (u + dt L(u)) and 1/3 f^n + 2/3 (u + dt L(u))
-    const T cb = stage == 1 ? T(1) : (stage == 2 ? T(0.25) : T(2.0 / 3.0));
-    // warp p of a group of G populations also evaluates the faces on the
-    // tile's right and top edges for the group's p-th population:
-    // lane l < TY: x-face right of node (TX-1, l); every lane: y-face above (l, TY-1)
-    const int ex_row = tx < TY ? tx : TY - 1;
-    // per-thread bases in the staged tile (all stencil offsets are immediates)
-    const int cidx = (ty + 3) * HXP + tx + 4;           // the node itself
-    const int xrow = (ty + 3) * HXP + tx;                // row of the node, column tx
-    const int ycol = ty * HXP + tx + 4;                  // column of the node, row ty
-    const int exrow = (ex_row + 3) * HXP + TX;           // extra x-face: virtual node (TX, ex_row)
-    const int eycol = TY * HXP + tx + 4;                 // extra y-face: virtual node (tx, TY)
 
-    for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int li = find_lattice(g.item_begin, n_lat, item);
-        const LatDesc* dp = g.desc + li;
-        if ((long long)j >= dp->remaining) {
-            item = last_item_of(*dp, item);
-            continue;
-        }
-        const int nx = dp->nx, ny = dp->ny, pitch = dp->pitch;
-        const long long plane = dp->plane;
-        const int local = item - dp->item_begin;
-        const int bx = local % dp->tiles_x, by = local / dp->tiles_x;
-        const int x0 = bx * TX, y0 = by * TY;
-        const int x = x0 + tx, y = y0 + ty;
-        const bool active = x < nx && y < ny;
-        const T* __restrict__ U = static_cast<const T*>(dp->buf[in_idx]);
-        const T* __restrict__ Fn = static_cast<const T*>(dp->buf[0]);
-        T* __restrict__ out = static_cast<T*>(dp->buf[out_idx]);
-        const T r0 = lat_val<T>(dp->rho0, dp->rho0_f);
-        const T cdx = lat_val<T>(dp->cdx, dp->cdx_f);
-        const T dtt = lat_val<T>(dp->dt_tau, dp->dt_tau_f);
-        const V eps = P::sp(lat_val<T>(dp->eps, dp->eps_f) * T(12.0 / 13.0));
-        const long long cell = (long long)y * pitch + x;
-        const bool interior = x0 >= 4 && x0 + TX + 4 <= nx && y0 >= 3 && y0 + TY + 3 <= ny;
-        // 16-byte asynchronous copies of the K halo tiles: a thread owns one
-        // (row, 16-byte column chunk) of the tile and copies it for every
-        // SK-th population, stepping by whole planes (no index arithmetic per
-        // copy); row_src(r, c) is the source of population 0
-        auto stage_rows16 = [&](int t, auto row_src) {
-            constexpr int CHUNKS = HY * RV;   // (row, 16-byte chunk) positions of a tile
-            if constexpr (NT >= CHUNKS) {
-                constexpr int SK = NT / CHUNKS;
-                if (t < SK * CHUNKS) {
-                    const int pr = t % CHUNKS, k0 = t / CHUNKS;
-                    const int r = pr / RV, c = pr - r * RV;
-                    const T* sp = row_src(r, c) + k0 * plane;
-                    T* dp16 = tiles + k0 * HXY + r * HXP + c * VEC;
-#pragma unroll 4
-                    for (int k = k0; k < K; k += SK, sp += SK * plane, dp16 += SK * HXY)
-                        if (LBM_BC_NODE(dp, K, sp - U) && LBM_BC_NODE(dp, K, sp - U + VEC - 1)) cp_async16(dp16, sp);
+    if (warp >= NM) {
+        if constexpr (Ge::RA > 0) set_regs_dec<Ge::RA>();
+        // ---- preparing warps: look up the block's items, copy their tiles,
+        //      form their moments and outer faces, one item ahead of the march
+        const int aw = warp - NM, atid = tid - NM * 32;
+        auto live_item = [&](int item, int& li) {
+            // first item from `item` on whose lattice still has steps to run
+            // (`total` or beyond: none), and that lattice
+            for (; item < total; item += gridDim.x) {
+                li = 0;
+                int first = 0, end = total;
+                bool dead;
+                if (n_lat == 1) {
+                    dead = (long long)j >= s_desc[0].remaining;
+                } else if (n_lat <= LATS) {
+                    int hi = n_lat - 1;
+                    while (li < hi) {
+                        const int mid = (li + hi + 1) >> 1;
+                        if (s_begin[mid] <= item) li = mid;
+                        else hi = mid - 1;
+                    }
+                    first = s_begin[li];
+                    if (li + 1 < n_lat) end = s_begin[li + 1];
+                    dead = s_dead[li];
+                } else {
+                    li = find_lattice(g.item_begin, n_lat, item);
+                    first = g.desc[li].item_begin;
+                    end = first + g.desc[li].items;
+                    dead = (long long)j >= g.desc[li].remaining;
+                }
+                if (!dead) break;
+                item += (end - 1 - item) / (int)gridDim.x * (int)gridDim.x;   // passed over in one jump
+            }
+            return item;
+        };
+        // the item at or after `item` into slot s (one warp, asynchronous copy)
+        auto look_up = [&](int item, int s) {
+            int li = 0;
+            item = live_item(item, li);
+            if (lane == 0) s_item[s] = item;
+            if (item < total && lane < DCH)
+                cp_async16(reinterpret_cast<uint4*>(s_desc + s) + lane, reinterpret_cast<const uint4*>(g.desc + li) + lane);
+        };
+        constexpr int NIT = (RT * CH + 31) / 32;   // chunks of a population's tile per lane
+        if (aw == 0) look_up(blockIdx.x, 0);
+        cp_async_wait_all();
+        named_sync(1, NA * 32);
+        for (unsigned n = 0;; ++n) {
+            const int slot = n & 3;
+            const int b = NB == 2 ? n & 1 : 0;
+            T* const buf = bufs + b * Ge::buf;
+            T* const mo = buf + (size_t)K * PL;
+            T* const edges = mo + Ge::n_mom;
+            if (n >= NB) named_sync(4 + b, Ge::NT);
+            const int item = s_item[slot];
+            if (item >= total) {   // the march warps stop too
+                named_arrive(2 + b, Ge::NT);
+                if (NB == 2 && n >= 1) named_sync(4 + (1 - b), Ge::NT);
+                break;
+            }
+            const LatDesc* const cp = s_desc + slot;
+            const int local = item - cp->item_begin;
+            const int x0 = local % cp->tiles_x * TX, y0 = local / cp->tiles_x * TY;
+            const int nx = cp->nx, ny = cp->ny, pitch = cp->pitch;
+            const long long plane = cp->plane;
+            // 1. the K halo tiles of the stage input: 16-byte asynchronous
+            //    copies (interior rows are 16-byte aligned: x0 - 4 is a multiple
+            //    of 4, the pitch of 32; at the periodic edge no chunk straddles
+            //    the wrap point when nx is a multiple of VEC), else single
+            //    values. A lane copies the same chunks of every population's
+            //    tile: their offsets are formed once per item (below 2^32: a
+            //    plane's elements times the three buffers fit the device).
+            const T* const U0 = static_cast<const T*>(cp->buf[in_idx]);
+            const bool interior = x0 >= 4 && x0 + TX + 4 <= nx && y0 >= 3 && y0 + TY + 3 <= ny;
+            if (interior || nx % VEC == 0) {
+                unsigned so[NIT];
+#pragma unroll
+                for (int i = 0; i < NIT; ++i) {
+                    const int q = lane + 32 * i, r = q / CH, c = (q - r * CH) * VEC;
+                    const int y = y0 - 3 + r, x = x0 - 4 + c;
+                    so[i] = interior ? (unsigned)y * (unsigned)pitch + (unsigned)x
+                                     : (unsigned)wrap_near(y, ny) * (unsigned)pitch + (unsigned)wrap_near(x, nx);
+                }
+                for (int k = aw; k < K; k += NA) {
+                    const T* U = U0 + k * plane;
+                    T* t = buf + k * PL + lane * VEC;
+#pragma unroll
+                    for (int i = 0; i < NIT; ++i) {
+                        if ((i + 1) * 32 <= RT * CH || lane + 32 * i < RT * CH) {
+                            const T* s = U + so[i];
+                            if (LBM_BC_NODE(cp, K, s - U0) && LBM_BC_NODE(cp, K, s - U0 + VEC - 1)) cp_async16(t + 32 * VEC * i, s);
+                        }
+                    }
                 }
             } else {
-                for (int pr = t; pr < CHUNKS; pr += NT) {
-                    const int r = pr / RV, c = pr - r * RV;
-                    const T* sp = row_src(r, c);
-                    T* dp16 = tiles + r * HXP + c * VEC;
-#pragma unroll 4
-                    for (int k = 0; k < K; ++k, sp += plane, dp16 += HXY)
-                        if (LBM_BC_NODE(dp, K, sp - U) && LBM_BC_NODE(dp, K, sp - U + VEC - 1)) cp_async16(dp16, sp);
+                for (int k = aw; k < K; k += NA) {
+                    const T* U = U0 + k * plane;
+                    for (int i = lane; i < RT * HXP; i += 32) {
+                        const int r = i / HXP, c = i - r * HXP;
+                        const T* s = U + ((long long)wrap_near(y0 - 3 + r, ny) * pitch + wrap_near(x0 - 4 + c, nx));
+                        if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(buf + k * PL + i, s);
+                    }
+                }
+            }
+            // the next item's descriptor travels with the copies
+            if (aw == 0) look_up(item + gridDim.x, (n + 1) & 3);
+            const T r0 = lat_val<T>(cp->rho0, cp->rho0_f);
+            const V eps = P::sp(lat_val<T>(cp->eps, cp->eps_f) * T(0.75));
+            const bool obs = stage == 1 && observe_now(*cp, j);
+            cp_async_wait_all();
+            named_sync(1, NA * 32);
+            // population k at tile row r, column c (halo: negative and beyond
+            // TY, TX)
+            auto at = [&](int k, int r, int c) {
+                return buf + k * PL + (r + 3) * HXP + c + 4;
+            };
+            if constexpr (IMEX) {
+                // the implicit BGK part of the stage in closed form, at every
+                // staged node: the stage value Y solves Y = u + dt g C(Y), C(Y) =
+                // -(Y - f^eq(Y)) / tau; the collision conserves rho and rho u
+                // (Eq. herfeq has the moments of Eq. f_moments_discrete), so
+                // f^eq(Y) = f^eq(u) and Y = (u + lam f^eq(u)) / (1 + lam). Values
+                // in the storage form: the map is linear, the offsets carry over.
+                // lam = g dt/tau, il = 1/(1 + lam)
+                const V vlam = P::mulc(P::sp(lat_val<T>(cp->dt_tau, cp->dt_tau_f)), T(IMEX_GAMMA));
+                const V vil = P::sp(T(1) / P::get(P::add(P::sp(T(1)), vlam), 0));
+                for (int pos = atid; pos < RT * (HXP / N); pos += NA * 32) {
+                    const int r = pos / (HXP / N) - 3, c = pos % (HXP / N) * N - 4;
+                    V dr, jx, jy;
+                    set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c)); }, dr, jx, jy);
+                    Equil<T> e;
+                    e.set(P::add(P::sp(r0), dr), dr, jx, jy);
+                    const EquilAll<T, Q1> ea(e);
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const V geq = P::mulc(ea.over_w(k), (T)w_of<Q1>(k));
+                        T* u = at(k, r, c);
+                        stv(u, P::mul(P::fma(vlam, geq, ldv_again(u)), vil));
+                    }
+                }
+                named_sync(1, NA * 32);
+            }
+
+            // 2. per warp, one of: the moments of a row of each group (Eq.
+            //    f_moments_discrete) with the observables of the state; the
+            //    faces beyond the outermost lane, one (population, rows) per lane
+            T acc[NOBS] = {T(0), T(0), T(0), T(0)};
+            constexpr int NE = (K * H + 31) / 32;
+            for (int task = aw; task < H + NE; task += NA) {
+                if (task < H) {
+                    const int r = task + grp * H;   // tile row
+                    V dr, jx, jy;
+                    set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c0)); }, dr, jx, jy);
+                    const V rho = P::add(P::sp(r0), dr);
+                    if (obs && y0 + r < ny) {
+                        const int pc = cp->probe_comp, y = y0 + r;
+#pragma unroll
+                        for (int h = 0; h < N; ++h) {
+                            const int x = x0 + c0 + h;
+                            if (x < nx) {
+                                acc[0] += P::get(dr, h);
+                                acc[1] += P::get(jx, h);
+                                acc[2] += P::get(jy, h);
+                                if (pc >= 0) {
+                                    T pxv, pyv;
+                                    if constexpr (sizeof(T) == 4) {
+                                        pxv = cp->probe_pxf[x];
+                                        pyv = cp->probe_pyf[y];
+                                    } else {
+                                        pxv = cp->probe_px[x];
+                                        pyv = cp->probe_py[y];
+                                    }
+                                    acc[3] += (pc == 0 ? P::get(jx, h) : P::get(jy, h)) / P::get(rho, h) * pxv * pyv;
+                                }
+                            }
+                        }
+                    }
+                    Equil<T> e;
+                    e.set(rho, dr, jx, jy);
+                    // FP32: residual moments of the collision term. In exact
+                    // arithmetic sum_k (u_k - geq_k) (1, v_k) = 0; in float32 the
+                    // rounding of the moments and of geq leaves a residual of
+                    // ~1e-7 of the momentum per stage, which is not small next to
+                    // the viscous decay per stage of a slowly decaying flow. It is
+                    // computed from the differences u_k - geq_k (accurate) and
+                    // removed with w_k (R0 + v_k . R1), which has exactly these
+                    // moments (quadrature identities of the set): the linear part
+                    // of the equilibrium takes the shifted moments dr + R0, j + R1.
+                    if constexpr (sizeof(T) == 4) {
+                        const T* U = static_cast<const T*>(cp->buf[in_idx]) + ((long long)(y0 + r) * pitch + x0 + c0);
+                        const bool in = y0 + r < ny && x0 + c0 < nx;
+                        const EquilAll<T, Q1> ea(e);
+                        V R0, R1x, R1y;
+                        set_moments<T, Q1>(
+                            [&](int k) {
+                                const V ew = ea.over_w(k);
+                                V u;
+                                if constexpr (IMEX)   // the stage input (the tile holds the stage values)
+                                    u = in && LBM_BC_NODE(cp, K, U - static_cast<const T*>(cp->buf[in_idx]) + k * plane)
+                                            ? ldv(U + k * plane) : P::sp(T(0));
+                                else
+                                    u = ldv_again(at(k, r, c0));
+                                return P::fmac(ew, -(T)w_of<Q1>(k), u);
+                            },
+                            R0, R1x, R1y);
+                        e.e0 = P::add(e.e0, R0);
+                        e.jx = P::add(e.jx, R1x);
+                        e.jy = P::add(e.jy, R1y);
+                    }
+                    T* m = mo + 2 * (r * TX + c0);
+                    stv2(m, e.px, e.py);
+                    stv2(m + 2 * TY * TX, e.jx, e.jy);
+                    stv(mo + 4 * TY * TX + r * TX + c0, e.e0);
+                } else {
+                    const int q = (task - H) * 32 + lane;
+                    const int k = q / H, r = q - k * H;   // march row (of each group)
+                    if (k < K && (Q1 % 2 == 0 || 2 * (k % Q1) + 1 != Q1)) {
+                        const bool mx = 2 * (k % Q1) + 1 < Q1;
+                        const int st = mx ? -1 : 1;
+                        const bool my = 2 * (k / Q1) + 1 < Q1;
+                        const T* a = buf + k * PL + (my ? RT - 4 - r : r + 3) * HXP + (mx ? 6 : TX + 1);
+                        const T* b = a + (my ? 1 - N : N - 1) * H * HXP;
+                        const V f = weno5_vals<P, T>(P::mk(a[0], b[0]), P::mk(a[st], b[st]), P::mk(a[2 * st], b[2 * st]),
+                                                     P::mk(a[3 * st], b[3 * st]), P::mk(a[4 * st], b[4 * st]), eps);
+                        edges[k * TY + r] = P::get(f, 0);
+                        edges[k * TY + r + (N - 1) * H] = P::get(f, N - 1);
+                    }
+                }
+            }
+            if (obs) {
+                // fixed order: lanes, then warps
+#pragma unroll
+                for (int q = 0; q < NOBS; ++q) {
+                    T v = acc[q];
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if (lane == 0) red[aw * NOBS + q] = (double)v;
+                }
+                named_sync(1, NA * 32);
+                if (atid < NOBS) {
+                    double s = 0.0;
+                    for (int w = 0; w < NA; ++w) s += red[w * NOBS + atid];
+                    cp->partials[(long long)local * NOBS + atid] = s;
+                }
+            }
+            named_arrive(2 + b, Ge::NT);
+        }
+        return;
+    }
+
+    if constexpr (Ge::RM > 0) set_regs_inc<Ge::RM>();
+    // ---- march warps
+    // stage weights: f^(s) = f^n + cb ((u - f^n) + dt L(u)), i.e. the Shu-Osher
+    // combinations 3/4 f^n + 1/4 (u + dt L(u)) and 1/3 f^n + 2/3 (u + dt L(u))
+    const V cb = P::sp(stage == 1 ? T(1) : (stage == 2 ? T(0.25) : T(2.0 / 3.0)));
+    for (unsigned n = 0;; ++n) {
+        const int slot = n & 3;
+        const int b = NB == 2 ? n & 1 : 0;
+            T* const buf = bufs + b * Ge::buf;
+        const T* const mom = buf + (size_t)K * PL;
+        const T* const edges = mom + Ge::n_mom;
+        named_sync(2 + b, Ge::NT);
+        const int item = s_item[slot];
+        if (item >= total) break;
+        const LatDesc* const cp = s_desc + slot;
+        const int local = item - cp->item_begin;
+        const int x0 = local % cp->tiles_x * TX, y0 = local / cp->tiles_x * TY;
+        const int nx = cp->nx, ny = cp->ny, pitch = cp->pitch;
+        const long long plane = cp->plane;
+        const T cdx = lat_val<T>(cp->cdx, cp->cdx_f);
+        const T dtt = lat_val<T>(cp->dt_tau, cp->dt_tau_f);
+        const V eps = P::sp(lat_val<T>(cp->eps, cp->eps_f) * T(0.75));
+        // IMEX: (dt/tau) / (1 + lam)
+        [[maybe_unused]] const T c1 = dtt / P::get(P::add(P::sp(T(1)), P::mulc(P::sp(dtt), T(IMEX_GAMMA))), 0);
+
+        auto march = [&](auto sx_, auto full_, int k, int seg, const T* tk) {
+            constexpr int SX = decltype(sx_)::value;
+            constexpr bool FULL = decltype(full_)::value;   // every node of the tile is inside the lattice
+            const T svx = c_set<T, Q1>.vx[k], svy = c_set<T, Q1>.vy[k];
+            const bool my = svy < T(0);
+            const bool movy = Q1 % 2 == 0 || svy != T(0);
+            const V vx = P::sp(svx), vy = P::sp(svy), w = P::sp(c_set<T, Q1>.w[k]);
+            const V cvx = P::sp((SX < 0 ? -svx : svx) * cdx), cvy = P::sp((my ? -svy : svy) * cdx);
+            const V vdtt = P::sp(IMEX ? c1 : dtt);
+            const bool outer = lane % LC == (SX > 0 ? LC - 1 : 0);
+            const int rs = my ? -HXP : HXP;           // row stride of the march
+            const int t0 = grp * H + seg * HS;        // rows before the march's first, in its direction
+            tk += (my ? RT - 1 - t0 : t0) * HXP + c0;   // march row -3, column -4 of the lane's nodes
+            const T* ek = edges + k * TY + t0;
+            const int yt = my ? TY - 1 - t0 : t0;     // tile row of march row 0
+            const T* mp = mom + 2 * (yt * TX + c0);
+            const T* mp0 = mom + 4 * TY * TX + yt * TX + c0;
+            const int ms = my ? -TX : TX;
+            const int x = x0 + c0;
+            const long long off = k * plane + (long long)(y0 + yt) * pitch + x;
+            const long long os = my ? -pitch : pitch;
+            // node pointers, stepped row by row: f^n (RK3) or the stage input
+            // (IMEX), the output, IMEX P
+            const T* fp = static_cast<const T*>(cp->buf[IMEX ? in_idx : 0]) + off;
+            T* op = static_cast<T*>(cp->buf[out_idx]) + off;
+            [[maybe_unused]] T* pp = static_cast<T*>(cp->buf[2]) + off;
+            [[maybe_unused]] const T* pp_in = pp;
+            // march rows inside the lattice, one bit each (none beyond nx)
+            unsigned rows;
+            {
+                const int n = my ? TY - (ny - y0) - t0 : ny - y0 - t0;   // first row / row count
+                const int m = n < 0 ? 0 : (n > HS ? HS : n);
+                rows = x < nx ? (my ? ~((1u << m) - 1u) : (1u << m) - 1u) : 0u;
+            }
+            const bool two = N == 2 && x + 1 < nx;
+            auto load_nodes = [&](const T* p, int r) {
+                if ((FULL || ((rows >> r) & 1u)) && LBM_BC_NODE(cp, K, off + r * os)) return ldg_v(p);   // beyond nx: row padding, not used
+                return P::sp(T(0));
+            };
+            auto store_nodes = [&](T* p, int r, V v) {
+                if ((FULL || ((rows >> r) & 1u)) && LBM_BC_NODE(cp, K, off + r * os)) {
+                    if (FULL || N == 1 || two) stg_v(p, v);
+                    else stg_1(p, P::get(v, 0));
+                }
+            };
+            // rows unrolled: all of them, or two where the copies for the signs
+            // of v_x (three with an odd set) would outgrow the instruction cache
+            constexpr int UN = IMEX && Q1 == 4 ? HS : (Q1 == 3 && HS > 2 ? 2 : (Q1 == 5 && HS > 4 ? 2 : HS));
+            // the node values are loaded AH rows ahead of their use
+            constexpr int AH = Q1 == 4 ? (IMEX ? (HS < 2 ? HS : 2) : HS) : UN;
+            V fq[AH];
+            [[maybe_unused]] V pq[IMEX ? AH : 1];
+#pragma unroll
+            for (int r = 0; r < AH; ++r) {
+                fq[r] = node_in ? load_nodes(fp, r) : P::sp(T(0));
+                if constexpr (IMEX) pq[r] = stage == 2 ? load_nodes(pp_in, r) : P::sp(T(0));
+                fp += os;
+                if constexpr (IMEX) pp_in += os;
+            }
+            // face below march row 0
+            V dy1 = P::sp(T(0)), dy2 = dy1, dy3 = dy1, fy2 = dy1, top = dy1, last = dy1;
+            if (movy) {
+                const V a = ldv(tk + 4), b = ldv(tk + rs + 4), c = ldv(tk + 2 * rs + 4), d = ldv(tk + 3 * rs + 4);
+                last = ldv(tk + 4 * rs + 4);
+                const V d1 = P::sub(a, b);
+                dy1 = P::sub(b, c);
+                dy2 = P::sub(c, d);
+                dy3 = P::sub(d, last);
+                fy2 = weno5_f<P, T>(dy2, eps);
+                top = weno5_diff<P, T>(d1, dy1, dy2, dy3, weno5_f<P, T>(dy1, eps), fy2);
+            }
+            const T *tr = tk + 3 * rs, *ty = tk + 5 * rs + 4;   // the node's row; two rows ahead, the lane's column
+#pragma unroll (UN)
+            for (int r = 0; r < HS; ++r, mp += 2 * ms, mp0 += ms, op += os, tr += rs, ty += rs) {
+                const V fcur = fq[r % AH];
+                [[maybe_unused]] V pcur = P::sp(T(0));
+                if constexpr (IMEX) pcur = pq[r % AH];
+                if (r + AH < HS) {
+                    if (node_in) fq[r % AH] = load_nodes(fp, r + AH);
+                    fp += os;
+                    if constexpr (IMEX) {
+                        if (stage == 2) pq[r % AH] = load_nodes(pp_in, r + AH);
+                        pp_in += os;
+                    }
+                }
+                V uk, fl, dcx;
+                if constexpr (SX != 0) {
+                    V d1, d2, d4;
+                    uk = x_diffs<SX>(tr, d1, d2, dcx, d4);
+                    fl = weno5_diff<P, T>(d1, d2, dcx, d4, weno5_f<P, T>(d2, eps), weno5_f<P, T>(dcx, eps));
+                } else {
+                    uk = ldv(tr + 4);
+                }
+                Equil<T> e;
+                ldv2(mp, e.px, e.py);
+                ldv2(mp + 2 * TY * TX, e.jx, e.jy);
+                e.e0 = ldv(mp0);
+                const V ew = e.over_w(vx, vy);
+                // dt L(u)_k = -(dt/dx) v . dF - (u - geq) dt/tau; IMEX: dt C(Y)
+                // of the stage input u at the node
+                const V dtc = P::mulr(P::fma(w, ew, P::neg(IMEX ? fcur : uk)), vdtt);
+                V inc = IMEX ? P::sp(T(0)) : dtc;
+                if (movy) {
+                    const V nw = ldv(ty);
+                    const V dy4 = P::sub(last, nw);
+                    last = nw;
+                    const V fy3 = weno5_f<P, T>(dy3, eps);
+                    const V up = weno5_diff<P, T>(dy1, dy2, dy3, dy4, fy2, fy3);
+                    // flux difference (f_i - f_{i-1}) + (d_{i+1/2} - d_{i-1/2})/3
+                    // (negated): the upwind node values differ by one node
+                    // (exact for close values), the corrections d are small
+                    inc = P::fma(cvy, P::fmac(P::sub(top, up), T(1.0 / 3.0), dy2), inc);
+                    top = up;
+                    dy1 = dy2;
+                    dy2 = dy3;
+                    dy3 = dy4;
+                    fy2 = fy3;
+                }
+                if constexpr (SX != 0) {
+                    const V fh = x_next<SX>(fl, ek[r], outer);
+                    inc = P::fma(cvx, P::fmac(P::sub(fl, fh), T(1.0 / 3.0), dcx), inc);
+                }
+                if constexpr (!IMEX) {
+                    // stage combination in increment form: one rounding of the
+                    // stored value per stage (u - f^n is exact for close values);
+                    // stage 1: u + dt L(u) (fcur is 0, cb 1)
+                    store_nodes(op, r, P::fma(cb, P::add(P::sub(uk, fcur), inc), fcur));
+                } else if (stage == 1) {
+                    store_nodes(op, r, P::add(fcur, P::fmac(dtc, T(1.0 - 2.0 * IMEX_GAMMA), inc)));   // Z
+                    store_nodes(pp, r, P::fmac(dtc, T(2.0 * IMEX_GAMMA), fcur));                       // P
+                    pp += os;
+                } else {
+                    store_nodes(op, r, P::fmac(P::add(P::sub(fcur, pcur), P::add(inc, dtc)), T(0.5), pcur));
                 }
             }
         };
-
-        // 1. stage all K halo tiles of the stage input
-        __syncthreads();  // the previous item is done with the tiles (and s_obs)
-        if (tid == 0) s_obs = stage == 1 && observe_now(*dp, j);
-        if (interior) {
-            // rows are 16-byte aligned (x0 - 4 is a multiple of 4, pitch of
-            // 32): every thread issues all its 16-byte asynchronous copies,
-            // then waits once
-            const T* src = U + (long long)(y0 - 3) * pitch + (x0 - 4);
-            stage_rows16(tid, [&](int r, int c) { return src + (long long)r * pitch + c * VEC; });
-            cp_async_wait_all();
-        } else {
-            // periodic edge: wrapped row offsets and columns once per tile,
-            // then asynchronous copies from the wrapped positions
-            for (int i = tid; i < HY + HXP; i += NT) {
-                if (i < HY) s_row[i] = (long long)wrapi(y0 - 3 + i, ny) * pitch;
-                else s_col[i - HY] = wrapi(x0 - 4 + (i - HY), nx);
-            }
-            __syncthreads();
-            if (nx % VEC == 0) {
-                // a 16-byte column chunk starts at a multiple of VEC and the
-                // wrap point nx is one, so no chunk straddles it: one copy
-                // per chunk from its wrapped start column
-                stage_rows16(tid, [&](int r, int c) { return U + s_row[r] + s_col[c * VEC]; });
-            } else {
-                for (int i = tid; i < K * HXY; i += NT) {
-                    const int k = i / HXY, rem = i - k * HXY;
-                    const int r = rem / HXP, c = rem - r * HXP;
-                    if (LBM_BC_NODE(dp, K, k * plane + s_row[r] + s_col[c]))
-                        cp_async_small<sizeof(T)>(tiles + i, U + k * plane + s_row[r] + s_col[c]);
-                }
-            }
-            cp_async_wait_all();
-        }
-        const T* __restrict__ fnp = (IMEX ? U : Fn) + cell;   // node values of f^n (RK3) / of the input (IMEX)
-        const T* __restrict__ ppn = static_cast<const T*>(dp->buf[2]) + cell;   // IMEX stage 2: P
-        T* __restrict__ pout = static_cast<T*>(dp->buf[2]) + cell;              // IMEX stage 1: P
-        // IMEX constants: lam = g dt/tau, il = 1/(1 + lam), c1 = (dt/tau) il
-        const T lam = T(IMEX_GAMMA) * dtt, il = T(1) / (T(1) + lam), c1 = dtt * il;
-        T* __restrict__ op = out + cell;
-        __syncthreads();
-        if constexpr (IMEX) {
-            imex_stage_values<T, Q1>(tiles, HXY, r0, lam, il, tid, NT);
-            __syncthreads();
-        }
-
-        // 2. moments of the stage input at this node, Eq. (f_moments_discrete)
-        //    (ascending k; FP32 with 16 velocities: through the column sums
-        //    over iy and the row sums over ix of the product set, fewer
-        //    operations)
-        T dr = T(0), jx = T(0), jy = T(0);
-        if constexpr (sizeof(T) == 4 && Q1 == 4) {
-            T cs[Q1], rs[Q1];
-            sum_cols_rows<T, Q1>([&](int k) { return tiles[k * HXY + cidx]; }, cs, rs);
-            moments_of_sums<T, Q1>(cs, rs, dr, jx, jy);
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const T u = tiles[k * HXY + cidx];
-                dr += u;
-                if (vx_of<Q1>(k) != 0.0) jx += u * (T)vx_of<Q1>(k);
-                if (vy_of<Q1>(k) != 0.0) jy += u * (T)vy_of<Q1>(k);
-            }
-        }
-        const T rho = r0 + dr;
-        const T inv = active ? T(1) / rho : T(0);
-        const T ux = jx * inv, uy = jy * inv;
-        const T usq = ux * ux + uy * uy;
-
-        if (s_obs) {
-            T acc[NOBS] = {T(0), T(0), T(0), T(0)};
-            if (active) {
-                acc[0] = dr;
-                acc[1] = jx;
-                acc[2] = jy;
-                const int pc = dp->probe_comp;
-                if (pc >= 0) {
-                    T pxv, pyv;
-                    if constexpr (sizeof(T) == 4) {
-                        pxv = dp->probe_pxf[x];
-                        pyv = dp->probe_pyf[y];
-                    } else {
-                        pxv = dp->probe_px[x];
-                        pyv = dp->probe_py[y];
-                    }
-                    acc[3] = (pc == 0 ? ux : uy) * pxv * pyv;
-                }
-            }
-            // no trailing barrier: `red` is next written after the next
-            // item's staging barrier
-            block_reduce_obs<T, NT, false>(acc, dp->partials + (long long)local * NOBS, red);
-        }
-
-        // FP32: residual moments of the collision term. In exact arithmetic
-        // sum_k (u_k - geq_k) (1, v_k) = 0; in float32 the rounding of the
-        // moments and of geq leaves a residual of ~1e-7 of the momentum per
-        // stage, which is not small next to the viscous decay per stage of a
-        // slowly decaying flow. It is computed from the differences u_k - geq_k
-        // (accurate) and removed below with w_k (R0 + v_k . R1), which has
-        // exactly these moments (quadrature identities of the set).
-        // The stored equilibrium is written w_k (dr + v_k . j + rho/2 ((v_k . u)^2
-        // - u^2)), i.e. Eq. (herfeq) minus w_k rho0 with rho (v_k . u) = v_k . j.
-        const T hr = T(0.5) * rho;
-        T R0 = T(0), R1x = T(0), R1y = T(0);
-        if constexpr (sizeof(T) == 4) {
-            // v_k . u and v_k . j + dr from per-axis terms (v_x u_x for each
-            // node of the 1D set, v_y u_y + ... for each row of the product set)
-            const EqTerms<T, Q1> e{ux, uy, jx, jy, dr};
-            auto dk = [&](int k) {
-                T geq;
-                if constexpr (Q1 == 4) {
-                    const T xi = e.xi(k);
-                    geq = (T)w_of<Q1>(k) * (hr * (xi * xi - usq) + e.lin(k));
-                } else {
-                    const T vx = (T)vx_of<Q1>(k), vy = (T)vy_of<Q1>(k);
-                    const T xi = vx * ux + vy * uy;
-                    geq = (T)w_of<Q1>(k) * (hr * (xi * xi - usq) + (vx * jx + (vy * jy + dr)));
-                }
-                // the stage input at the node (IMEX: from global memory, the
-                // tile holds the stage values)
-                const T uin = IMEX ? ((active && LBM_BC_NODE(dp, K, cell + k * plane)) ? fnp[k * plane] : T(0))
-                                   : tiles[k * HXY + cidx];
-                return uin - geq;
+        const bool full_tile = x0 + TX <= nx && y0 + TY <= ny;
+#pragma unroll 1
+        for (int m = warp; m < K * S; m += NM) {
+            const int k = S == 1 ? m : m % K, seg = S == 1 ? 0 : m / K;
+            const T* tk = buf + k * PL;
+            auto by_sign = [&](auto full_) {
+                if (Q1 % 2 == 1 && 2 * (k % Q1) + 1 == Q1) march(Const<0>{}, full_, k, seg, tk);
+                else if (2 * (k % Q1) + 1 < Q1) march(Const<-1>{}, full_, k, seg, tk);
+                else march(Const<1>{}, full_, k, seg, tk);
             };
-            if constexpr (Q1 == 4) {
-                // sums through the columns and rows of the product set
-                T cs[Q1], rs[Q1];
-                sum_cols_rows<T, Q1>(dk, cs, rs);
-                moments_of_sums<T, Q1>(cs, rs, R0, R1x, R1y);
-            } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const T d = dk(k);
-                    R0 += d;
-                    if (vx_of<Q1>(k) != 0.0) R1x += d * (T)vx_of<Q1>(k);
-                    if (vy_of<Q1>(k) != 0.0) R1y += d * (T)vy_of<Q1>(k);
-                }
-            }
+            if (full_tile) by_sign(Const<1>{});
+            else by_sign(Const<0>{});
         }
-        // the correction w_k (R0 + v_k . R1) enters the equilibrium as
-        // shifted moments: dr + R0, j + R1
-        const T drc = dr + R0, jxc = jx + R1x, jyc = jy + R1y;
-        const EqTerms<T, Q1> ec{ux, uy, jxc, jyc, drc};
-
-        // 3. per group of G populations: every thread evaluates the x- and
-        //    y-face on the low side of its node for each population of the
-        //    group (one packed pair each), the tile's right- and top-edge
-        //    faces are added (below), one barrier, then every node updates
-        //    those G populations from the four faces around it. Two face
-        //    buffers alternate between groups; with one, a barrier also
-        //    precedes each group's faces. With the 16-velocity set the packed
-        //    pairs are two populations' x-faces and then their y-faces instead
-        //    of one population's x- and y-face, and faces are stored and read
-        //    back as pairs (half the shared-memory instructions for them); its
-        //    edge faces are evaluated through one copy of the code for all the
-        //    group's pairs (an unrolled copy per pair and axis had made the
-        //    kernel's instructions outgrow the instruction cache: the warps
-        //    stalled on instruction fetch), the x-edges of all pairs packed one
-        //    (pair, row) per lane.
-#pragma unroll
-        for (int k0 = 0; k0 < K; k0 += G) {
-            T* fg = faces + (FB == 2 ? ((k0 / G) & 1) * G * NF : 0);
-            if (FB == 1 && k0 > 0) __syncthreads();  // the previous group's update is done with the faces
-            T fnv[G];
-            T pv[IMEX ? G : 1];   // IMEX stage 2: P at the node
-            if constexpr (PAIRS) {
-                // populations 2q and 2q+1 of the group side by side: the x-faces
-                // of both as one packed pair, then the y-faces of both; faces
-                // stored as pairs [TY][TX + 1] and [TY + 1][TX] of V per q
-#pragma unroll
-                for (int q = 0; q < G / 2; ++q) {
-                    const int ka = k0 + 2 * q;
-                    const T* ta = tiles + ka * HXY;
-                    const T* tb = ta + HXY;
-                    V* fx2 = reinterpret_cast<V*>(fg) + q * NF;
-                    V* fy2 = fx2 + NFX;
-                    const double vxd = vx_of<Q1>(ka), vyd = vy_of<Q1>(ka);   // also the signs of ka + 1
-                    const int xo = vxd > 0 ? 1 : 6, xs = vxd > 0 ? 1 : -1;
-                    const int yo = vyd > 0 ? 0 : 5 * HXP, ys = vyd > 0 ? HXP : -HXP;
-                    auto face = [&](int base, int o, int st) {
-                        const T* a = ta + base + o;
-                        const T* b = tb + base + o;
-                        return weno5_pair<T>(P::mk(a[0], b[0]), P::mk(a[st], b[st]), P::mk(a[2 * st], b[2 * st]),
-                                             P::mk(a[3 * st], b[3 * st]), P::mk(a[4 * st], b[4 * st]), eps);
-                    };
-                    fx2[ty * (TX + 1) + tx] = face(xrow, xo, xs);
-                    fy2[ty * TX + tx] = face(ycol, yo, ys);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int k = ka + h;
-                        fnv[2 * q + h] = (node_in && active && LBM_BC_NODE(dp, K, cell + k * plane)) ? fnp[k * plane] : T(0);
-                        if constexpr (IMEX)
-                            pv[2 * q + h] = (stage == 2 && active && LBM_BC_NODE(dp, K, cell + k * plane)) ? ppn[k * plane] : T(0);
-                    }
-                }
-                // the tile's right-edge x-faces and top-edge y-faces of the
-                // group's pairs, through one copy of the code (pair and stencil
-                // direction selected at run time): edge tasks e < NXE are the
-                // right-edge x-faces of all pairs and rows, one (pair, row) per
-                // lane; task NXE + q is pair q's top-edge y-faces, one column
-                // per lane; task e is evaluated by warp e mod TY
-                constexpr int NPR = G / 2;
-                constexpr int NXE = (NPR * TY + 31) / 32;
-                for (int e = ty; e < NXE + NPR; e += TY) {
-                    const bool xax = e < NXE;
-                    const int lx = e * 32 + tx;                    // x task: (pair, row) of this lane
-                    const bool xok = lx < NPR * TY;
-                    const int q = xax ? (xok ? lx / TY : 0) : e - NXE;
-                    const int row = xax ? (xok ? lx % TY : 0) : 0;
-                    const T* ta = tiles + (k0 + 2 * q) * HXY;
-                    const T* tb = ta + HXY;
-                    V* fx2 = reinterpret_cast<V*>(fg) + q * NF;
-                    // pair q's nodes along x are (2q mod Q1, +1): both below the
-                    // middle of the 1D set (v_x < 0) or both above (v_x > 0);
-                    // v_y has one sign in the whole group (whole rows)
-                    const bool xpos = 2 * ((2 * q) % Q1) >= Q1;
-                    const bool ypos = vy_of<Q1>(k0) > 0;
-                    const int st = xax ? (xpos ? 1 : -1) : (ypos ? HXP : -HXP);
-                    const int base = xax ? (row + 3) * HXP + TX + (xpos ? 1 : 6) : eycol + (ypos ? 0 : 5 * HXP);
-                    const T* a = ta + base;
-                    const T* b = tb + base;
-                    const V f = weno5_pair<T>(P::mk(a[0], b[0]), P::mk(a[st], b[st]), P::mk(a[2 * st], b[2 * st]),
-                                              P::mk(a[3 * st], b[3 * st]), P::mk(a[4 * st], b[4 * st]), eps);
-                    if (xax) {
-                        if (xok) fx2[row * (TX + 1) + TX] = f;
-                    } else {
-                        fx2[NFX + TY * TX + tx] = f;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int p = 0; p < G; ++p) {
-                    const int k = k0 + p;
-                    if (k >= K) break;
-                    const T* tk = tiles + k * HXY;
-                    T* fx = fg + p * NF;            // [TY][TX + 1]
-                    T* fy = fx + NFX;               // [TY + 1][TX]
-                    const double vxd = vx_of<Q1>(k), vyd = vy_of<Q1>(k);
-                    // upwind stencil of the face on the low side of node (c, r):
-                    // x, v > 0: cols c+1..c+5 of row r+3; v < 0: cols c+6..c+2
-                    // y, v > 0: rows r..r+4 of col c+4; v < 0: rows r+5..r+1
-                    const int xo = vxd > 0 ? 1 : 6, xs = vxd > 0 ? 1 : -1;
-                    const int yo = vyd > 0 ? 0 : 5 * HXP, ys = vyd > 0 ? HXP : -HXP;
-                    {
-                        const T* px = tk + xrow + xo;
-                        const T* py = tk + ycol + yo;
-                        const V f = weno5_pair<T>(P::mk(px[0], py[0]), P::mk(px[xs], py[ys]), P::mk(px[2 * xs], py[2 * ys]),
-                                                  P::mk(px[3 * xs], py[3 * ys]), P::mk(px[4 * xs], py[4 * ys]), eps);
-                        fx[ty * (TX + 1) + tx] = f.x;
-                        fy[ty * TX + tx] = f.y;
-                    }
-                    if (ty == p % TY) {
-                        const T* px = tk + exrow + xo;
-                        const T* py = tk + eycol + yo;
-                        const V f = weno5_pair<T>(P::mk(px[0], py[0]), P::mk(px[xs], py[ys]), P::mk(px[2 * xs], py[2 * ys]),
-                                                  P::mk(px[3 * xs], py[3 * ys]), P::mk(px[4 * xs], py[4 * ys]), eps);
-                        if (tx < TY) fx[tx * (TX + 1) + TX] = f.x;
-                        fy[TY * TX + tx] = f.y;
-                    }
-                    fnv[p] = (node_in && active && LBM_BC_NODE(dp, K, cell + k * plane)) ? fnp[k * plane] : T(0);
-                    if constexpr (IMEX)
-                        pv[p] = (stage == 2 && active && LBM_BC_NODE(dp, K, cell + k * plane)) ? ppn[k * plane] : T(0);
-                }
-            }
-            __syncthreads();
-            if (active) {
-                V pxl, pxr, pyb, pyt;   // face pairs of populations 2q, 2q+1 (PAIRS)
-#pragma unroll
-                for (int p = 0; p < G; ++p) {
-                    const int k = k0 + p;
-                    if (k >= K) break;
-                    const T* tk = tiles + k * HXY;
-                    const T* fx = fg + p * NF;
-                    const T* fy = fx + NFX;
-                    const double vxd = vx_of<Q1>(k), vyd = vy_of<Q1>(k);
-                    // the four faces around the node: low/high x, low/high y
-                    T fxl, fxh, fyl, fyh;
-                    if constexpr (PAIRS) {
-                        if ((p & 1) == 0) {
-                            const V* fx2 = reinterpret_cast<const V*>(fg) + (p >> 1) * NF;
-                            const V* fy2 = fx2 + NFX;
-                            pxl = fx2[ty * (TX + 1) + tx];
-                            pxr = fx2[ty * (TX + 1) + tx + 1];
-                            pyb = fy2[ty * TX + tx];
-                            pyt = fy2[(ty + 1) * TX + tx];
-                        }
-                        fxl = (p & 1) ? pxl.y : pxl.x;
-                        fxh = (p & 1) ? pxr.y : pxr.x;
-                        fyl = (p & 1) ? pyb.y : pyb.x;
-                        fyh = (p & 1) ? pyt.y : pyt.x;
-                    } else {
-                        fxl = fx[ty * (TX + 1) + tx];
-                        fxh = fx[ty * (TX + 1) + tx + 1];
-                        fyl = fy[ty * TX + tx];
-                        fyh = fy[(ty + 1) * TX + tx];
-                    }
-                    // flux difference F(i+1/2) - F(i-1/2) = (c+ - c-) + (d+ - d-)/12:
-                    // the upwind node values c differ by one node (exact for
-                    // close values), the stored corrections d = 12 (face - c) are small
-                    const T vx = (T)vxd, vy = (T)vyd;
-                    const T uk = tk[cidx];
-                    // a = v_x dF_x + v_y dF_y (zero components drop out)
-                    T a = T(0);
-                    if (vxd != 0.0) {
-                        const T dc = vxd > 0 ? uk - tk[cidx - 1] : tk[cidx + 1] - uk;
-                        a = vx * ((fxh - fxl) * T(1.0 / 12.0) + dc);
-                    }
-                    if (vyd != 0.0) {
-                        const T dc = vyd > 0 ? uk - tk[cidx - HXP] : tk[cidx + HXP] - uk;
-                        a += vy * ((fyh - fyl) * T(1.0 / 12.0) + dc);
-                    }
-                    T xi, geq;
-                    if constexpr (sizeof(T) == 4 && Q1 == 4) {
-                        xi = ec.xi(k);
-                        geq = (T)w_of<Q1>(k) * (hr * (xi * xi - usq) + ec.lin(k));
-                    } else {
-                        xi = vx * ux + vy * uy;
-                        geq = (T)w_of<Q1>(k) * (hr * (xi * xi - usq) + (vx * jxc + (vy * jyc + drc)));
-                    }
-                    if constexpr (IMEX) {
-                        // dt A(Y)_k and dt C(Y)_k (from the stage input at the node)
-                        const T dta = -(a * cdx);
-                        const T dtc = -(c1 * (fnv[p] - geq));
-                        if (LBM_BC_NODE(dp, K, cell + k * plane)) {
-                            if (stage == 1) {
-                                op[k * plane] = fnv[p] + (dta + T(1.0 - 2.0 * IMEX_GAMMA) * dtc);   // Z
-                                pout[k * plane] = fnv[p] + T(2.0 * IMEX_GAMMA) * dtc;             // P
-                            } else {
-                                op[k * plane] = pv[p] + T(0.5) * ((fnv[p] - pv[p]) + (dta + dtc));
-                            }
-                        }
-                    } else {
-                        // dt L(u)_k = -(dt/dx) a - (u - geq) dt/tau
-                        const T inc = (geq - uk) * dtt - a * cdx;
-                        // stage combination in increment form: one rounding of the
-                        // stored value per stage (u - f^n is exact for close values)
-                        if (LBM_BC_NODE(dp, K, cell + k * plane))
-                            op[k * plane] = stage == 1 ? uk + inc : fnv[p] + cb * ((uk - fnv[p]) + inc);
-                    }
-                }
-            }
-        }
+        named_arrive(4 + b, Ge::NT);
     }
 }
 
@@ -644,64 +807,53 @@ int fd_tile_ty(int v) {
     return 0;
 }
 
+// A kernel variant: its entry, block size, dynamic shared memory and, where
+// the warpgroups split the launch's registers, the registers of their shares.
+struct FdVariant {
+    const void* fn = nullptr;
+    int threads = 0;
+    size_t bytes = 0;
+    int regs = 0;
+};
+template <typename T, int Q1, int TY, bool IMEX>
+static FdVariant fd_variant_of() {
+    using Ge = FdGeo<T, Q1, TY, IMEX>;
+    return FdVariant{(const void*)fd_stage_kernel<T, Q1, TY, IMEX>, Ge::NT, Ge::bytes, 32 * (Ge::NM * Ge::RM + Ge::NA * Ge::RA)};
+}
 template <typename T, int Q1, bool IMEX>
-static const void* fd_kernel_ptr_q(int tile) {
+static FdVariant fd_variant_q(int tile) {
     switch (tile) {
-        case FD_T32x8: return (const void*)fd_stage_kernel<T, Q1, 8, IMEX>;
-        case FD_T32x4: return (const void*)fd_stage_kernel<T, Q1, 4, IMEX>;
-        case FD_T32x16: return (const void*)fd_stage_kernel<T, Q1, 16, IMEX>;
-        case FD_T32x2: return (const void*)fd_stage_kernel<T, Q1, 2, IMEX>;
+        case FD_T32x8: return fd_variant_of<T, Q1, 8, IMEX>();
+        case FD_T32x4: return fd_variant_of<T, Q1, 4, IMEX>();
+        case FD_T32x16: return fd_variant_of<T, Q1, 16, IMEX>();
+        case FD_T32x2: return fd_variant_of<T, Q1, 2, IMEX>();
     }
-    return nullptr;
+    return FdVariant{};
 }
-
 template <typename T, bool IMEX>
-static const void* fd_kernel_ptr(int tile, int q1) {
+static FdVariant fd_variant_t(int tile, int q1) {
     switch (q1) {
-        case 3: return fd_kernel_ptr_q<T, 3, IMEX>(tile);
-        case 4: return fd_kernel_ptr_q<T, 4, IMEX>(tile);
-        case 5: return fd_kernel_ptr_q<T, 5, IMEX>(tile);
+        case 3: return fd_variant_q<T, 3, IMEX>(tile);
+        case 4: return fd_variant_q<T, 4, IMEX>(tile);
+        case 5: return fd_variant_q<T, 5, IMEX>(tile);
     }
-    return nullptr;
+    return FdVariant{};
 }
-
-template <typename T, int Q1>
-static size_t fd_smem_q(int tile) {
-    switch (tile) {
-        case FD_T32x8: return fd_smem_bytes<T, Q1, 8>();
-        case FD_T32x4: return fd_smem_bytes<T, Q1, 4>();
-        case FD_T32x16: return fd_smem_bytes<T, Q1, 16>();
-        case FD_T32x2: return fd_smem_bytes<T, Q1, 2>();
-    }
-    return 0;
-}
-
-template <typename T>
-static size_t fd_smem(int tile, int q1) {
-    switch (q1) {
-        case 3: return fd_smem_q<T, 3>(tile);
-        case 4: return fd_smem_q<T, 4>(tile);
-        case 5: return fd_smem_q<T, 5>(tile);
-    }
-    return 0;
-}
-
-static const void* fd_fn(int precision, int tile, int q1, int scheme) {
+static FdVariant fd_variant(int precision, int tile, int q1, int scheme) {
     if (scheme == LBM_TS_IMEX)
-        return precision == LBM_FP64 ? fd_kernel_ptr<double, true>(tile, q1) : fd_kernel_ptr<float, true>(tile, q1);
-    return precision == LBM_FP64 ? fd_kernel_ptr<double, false>(tile, q1) : fd_kernel_ptr<float, false>(tile, q1);
-}
-static size_t fd_bytes(int precision, int tile, int q1) {
-    return precision == LBM_FP64 ? fd_smem<double>(tile, q1) : fd_smem<float>(tile, q1);
+        return precision == LBM_FP64 ? fd_variant_t<double, true>(tile, q1) : fd_variant_t<float, true>(tile, q1);
+    return precision == LBM_FP64 ? fd_variant_t<double, false>(tile, q1) : fd_variant_t<float, false>(tile, q1);
 }
 
 // Opt each variant (both schemes' kernels) into the dynamic shared memory it
 // needs; once per process. A variant that cannot fit on this device is
 // refused (and the CUDA error state cleared).
 static cudaError_t fd_prepare(int precision, int tile, int q1) {
-    static int state[2][FD_NTILES][3] = {};  // 0 unknown, 1 ready, 2 does not fit
+    // 0 unknown, 1 ready, 2 does not fit; atomic: the two lanes of a server
+    // may prepare the same variant at once (both then make the same calls)
+    static std::atomic<int> state[2][FD_NTILES][3] = {};
     const int p = precision == LBM_FP64 ? 0 : 1;
-    int& st = state[p][tile][q1 - 3];
+    std::atomic<int>& st = state[p][tile][q1 - 3];
     if (st == 1) return cudaSuccess;
     if (st == 2) return cudaErrorInvalidConfiguration;
     int dev = 0, optin = 0;
@@ -710,15 +862,14 @@ static cudaError_t fd_prepare(int precision, int tile, int q1) {
         cudaGetLastError();
         return cudaErrorInvalidConfiguration;
     }
-    const size_t need = fd_bytes(precision, tile, q1);
-    if (need > (size_t)optin) {
-        st = 2;
-        return cudaErrorInvalidConfiguration;
-    }
     for (int scheme : {LBM_TS_RK3, LBM_TS_IMEX}) {
-        cudaError_t e = cudaFuncSetAttribute(fd_fn(precision, tile, q1, scheme),
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-        if (e != cudaSuccess) {
+        const FdVariant v = fd_variant(precision, tile, q1, scheme);
+        cudaFuncAttributes a;
+        if (v.bytes > (size_t)optin || cudaFuncGetAttributes(&a, v.fn) != cudaSuccess ||
+            // the shares must not exceed the registers the block is launched
+            // with (a warpgroup would wait for the rest for ever)
+            v.regs > (a.numRegs + 7) / 8 * 8 * v.threads ||
+            cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.bytes) != cudaSuccess) {
             cudaGetLastError();
             st = 2;
             return cudaErrorInvalidConfiguration;
@@ -735,13 +886,13 @@ cudaError_t launch_fd_stage(int precision, int q1, int scheme, int tile, int gri
         stage > fd_stages(scheme))
         return cudaErrorInvalidValue;
     if (scheme == LBM_TS_RK3_FUSED) return launch_fd_fused(precision, q1, tile, grid, g, j, s);
-    const void* fn = fd_fn(precision, tile, q1, scheme);
     cudaError_t e = fd_prepare(precision, tile, q1);
     if (e != cudaSuccess) return e;
+    const FdVariant v = fd_variant(precision, tile, q1, scheme);
     GroupDev gg = g;
     int jj = j, ss = stage;
     void* args[] = {&gg, &jj, &ss};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(fd_tile_tx(tile), fd_tile_ty(tile)), args, fd_bytes(precision, tile, q1), s);
+    return cudaLaunchKernel(v.fn, dim3(grid), dim3(v.threads), args, v.bytes, s);
 }
 
 bool fd_variant_fits(int precision, int q1, int tile, int scheme) {
@@ -752,11 +903,12 @@ bool fd_variant_fits(int precision, int q1, int tile, int scheme) {
 int fd_blocks_per_sm(int precision, int q1, int tile, int scheme) {
     if (scheme == LBM_TS_RK3_FUSED) return fd_fused_blocks_per_sm(precision, q1, tile);
     if (!fd_variant_fits(precision, q1, tile, scheme)) return 1;
+    const FdVariant v = fd_variant(precision, tile, q1, scheme);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fd_fn(precision, tile, q1, LBM_TS_RK3),
-                                                      fd_tile_tx(tile) * fd_tile_ty(tile),
-                                                      fd_bytes(precision, tile, q1)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v.fn, v.threads, v.bytes) != cudaSuccess) {
+        cudaGetLastError();
         return 1;
+    }
     return n > 0 ? n : 1;
 }
 

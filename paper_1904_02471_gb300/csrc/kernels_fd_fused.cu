@@ -12,8 +12,8 @@
 // for 32 x 8 tiles instead of 3).
 //
 // The arithmetic of every stage is that of the stage kernels (kernels_fd.cu):
-// the same WENO-5 interface values (12 (face - c), c the upwind node value),
-// flux differences (c+ - c-) + (d+ - d-)/12, BGK term with moments of the
+// the same WENO-5 interface values (3 (face - c), c the upwind node value),
+// flux differences (c+ - c-) + (d+ - d-)/3, BGK term with moments of the
 // stage input and, for FP32 deviation storage, the moment-exact collision
 // (residual moments of u - f^eq removed through shifted moments), and the
 // increment-form stage combinations f^n + cb ((u - f^n) + dt L(u)).
@@ -93,7 +93,7 @@ __device__ __forceinline__ typename Pr<T>::V fused_faces(const T* in, int W, int
     using P = Pr<T>;
     const int bx = R * W + (xp ? C - 3 : C + 2), sx = xp ? 1 : -1;
     const int by = (yp ? R - 3 : R + 2) * W + C, sy = yp ? W : -W;
-    return weno5_pair<T>(P::mk(in[bx], in[by]), P::mk(in[bx + sx], in[by + sy]), P::mk(in[bx + 2 * sx], in[by + 2 * sy]),
+    return weno5_vals<P, T>(P::mk(in[bx], in[by]), P::mk(in[bx + sx], in[by + sy]), P::mk(in[bx + 2 * sx], in[by + 2 * sy]),
                          P::mk(in[bx + 3 * sx], in[by + 3 * sy]), P::mk(in[bx + 4 * sx], in[by + 4 * sy]), eps);
 }
 
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
         const T rz = lat_val<T>(dp->rho0, dp->rho0_f);
         const T cdx = lat_val<T>(dp->cdx, dp->cdx_f);
         const T dtt = lat_val<T>(dp->dt_tau, dp->dt_tau_f);
-        const V eps = P::sp(lat_val<T>(dp->eps, dp->eps_f) * T(12.0 / 13.0));
+        const V eps = P::sp(lat_val<T>(dp->eps, dp->eps_f) * T(0.75));
         const bool interior = x0 >= 12 && x0 + 44 <= nx && y0 >= 9 && y0 + TY + 9 <= ny;
 
         __syncthreads();   // the previous item is done with shared memory
@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
             const T* fx = fxs + pp * Ge::FH * FW;
             const T* fy = fys + pp * Ge::FH * FW;
             T a = T(0);
-            if (vx != T(0)) a = vx * ((fx[r * FW + c + 1] - fx[r * FW + c]) * T(1.0 / 12.0) + dcx);
-            if (vy != T(0)) a += vy * ((fy[(r + 1) * FW + c] - fy[r * FW + c]) * T(1.0 / 12.0) + dcy);
+            if (vx != T(0)) a = vx * ((fx[r * FW + c + 1] - fx[r * FW + c]) * T(1.0 / 3.0) + dcx);
+            if (vy != T(0)) a += vy * ((fy[(r + 1) * FW + c] - fy[r * FW + c]) * T(1.0 / 3.0) + dcy);
             const T xi = vx * m.ux + vy * m.uy;
             const T geq = gc.w[pp] * (m.hr * (xi * xi - m.usq) + (vx * m.jxc + (vy * m.jyc + m.drc)));
             return (geq - uk) * dtt - a * cdx;
