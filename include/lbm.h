@@ -342,14 +342,15 @@ int lbm_batch_groups(lbm_batch* b, int* model, int* q, int* precision, int cap);
 /* Measurement: n steps launched one kernel at a time with CUDA events around
  * every kernel (no graph). ms[g*4 + k] (cap entries, caller-owned) receives
  * the summed device time of group g's kernels of kind k: 0..2 = CS step or FD
- * stages 1..3, 3 = observables finalisation; *total_ms the span of all n
- * steps. Computes exactly what lbm_batch_step(n) computes. Synchronous. */
+ * stages 1..3 (entry 3 stays 0: observables are recorded inside those
+ * kernels); *total_ms the span of all n steps. Computes exactly what lbm_batch_step(n) computes. Synchronous. */
 int lbm_batch_step_profiled(lbm_batch* b, int64_t n, double* ms, int cap, double* total_ms);
 
 /* Kernel configuration of group `group` of a batch (lbm_batch_groups order):
  * tile variant 0 .. lbm_n_tiles(model)-1 and grid size (blocks loop over the
- * group's work items; 0 picks the default: one block per work item, i.e. per
- * tile of every lattice of the group). Every variant computes bit-identical
+ * group's work items; 0 picks the default: for CS and the temporally blocked
+ * FD step one block per work item, i.e. per tile of every lattice of the
+ * group, for FD stages at most one block per SM). Every variant computes bit-identical
  * results; only speed differs. lbm_config does the same for a context. */
 int lbm_batch_config(lbm_batch* b, int group, int tile, int grid);
 int lbm_config(lbm_ctx* ctx, int tile, int grid);

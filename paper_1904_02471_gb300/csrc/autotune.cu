@@ -73,13 +73,10 @@ int Engine::tune(int trial_steps, std::string* report) {
         const int ntiles = g.model == LBM_CS ? (int)CS_NTILES : (int)FD_NTILES;
         float best = 1e30f;
         int best_tile = g.tile, best_grid = g.grid;
-        const int orig_any_obs = g.any_obs;
-        g.any_obs = false;
         for (int t = 0; t < ntiles; ++t) {
             if (g.model == LBM_FD && !fd_variant_fits(g.precision, g.q1, t, g.scheme)) continue;
             int rc = set_group_config(gi, t, 0);
             if (rc) return rc;
-            g.any_obs = false;
             const int full = g.total_items;
             const int pers = std::min(full, persistent_grid(g, t));
             const int cands[3] = {pers, std::min(full, 2 * pers), full};
@@ -124,7 +121,6 @@ int Engine::tune(int trial_steps, std::string* report) {
         }
         cudaStreamSynchronize(stream_);
         for (void* p : saved) cudaFree(p);
-        g.any_obs = orig_any_obs;
         int rc = set_group_config(gi, best_tile, best_grid);
         if (rc) return rc;
         {

@@ -18,6 +18,10 @@
 
 namespace lbm {
 
+// Tiles whose partial sums one block adds up (finish_obs).
+constexpr int OBS_GROUP = 256;
+__host__ __device__ constexpr long long obs_groups(long long items) { return (items + OBS_GROUP - 1) / OBS_GROUP; }
+
 constexpr int NOBS = 4;  // sum rho (minus the storage offset), sum j_x, sum j_y, probe sum
 
 struct alignas(16) LatDesc {   // copied in 16-byte chunks
@@ -48,6 +52,8 @@ struct alignas(16) LatDesc {   // copied in 16-byte chunks
     const float* probe_pxf;   // float copies for FP32 kernels
     const float* probe_pyf;
     double* partials;       // [items][NOBS], this lattice's slice
+    double* group_partials; // [obs_groups][NOBS]: sums of OBS_GROUP tiles each
+    unsigned* obs_count;    // [obs_groups + 1]: tiles done of each group, groups done (0 between launches)
     lbm_obs* series;        // [obs_cap]
     double* snap;           // [NOBS] result of a one-off observables reduction
     // float copies of omega, cdx, dt_tau, rho0, eps for the FP32 kernels (a
@@ -221,6 +227,90 @@ __device__ __forceinline__ void block_reduce_obs(const T (&v)[NOBS], double* out
         out[tid] = s;
     }
     if constexpr (TRAILING_SYNC) __syncthreads();
+}
+
+// The observables record of a state from its NOBS global sums.
+__device__ __forceinline__ lbm_obs make_obs(long long step, double dt, int nx, int ny, double rho0, int probe_comp,
+                                            double probe_norm, const double* tot) {
+    lbm_obs o;
+    o.step = step;
+    o.time = (double)step * dt;
+    o.mass = (double)nx * (double)ny * rho0 + tot[0];
+    o.mom_x = tot[1];
+    o.mom_y = tot[2];
+    o.amp = probe_comp >= 0 ? probe_norm * tot[3] : 0.0;
+    o.nonfinite = (isfinite(o.mass) && isfinite(o.amp) && isfinite(o.mom_x) && isfinite(o.mom_y)) ? 0 : 1;
+    o.reserved = 0;
+    return o;
+}
+
+// Sum of n rows of NOBS doubles by NT threads (fixed order): per-warp sums in
+// red[warp][NOBS] after a barrier.
+template <int NT, typename Sync>
+__device__ __forceinline__ void sum_partials(const double* p, int n, int tid, double* red, Sync sync) {
+    double a[NOBS] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = tid; i < n; i += NT) {
+        const double2 u = __ldcg(reinterpret_cast<const double2*>(p + (long long)i * NOBS));
+        const double2 v = __ldcg(reinterpret_cast<const double2*>(p + (long long)i * NOBS) + 1);
+        a[0] += u.x;
+        a[1] += u.y;
+        a[2] += v.x;
+        a[3] += v.y;
+    }
+#pragma unroll
+    for (int q = 0; q < NOBS; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+        if ((tid & 31) == 0) red[(tid >> 5) * NOBS + q] = a[q];
+    }
+    sync();
+}
+
+// Called by NT threads of a block (tid 0 .. NT - 1, `sync` a barrier of
+// theirs) after threads 0 .. NOBS - 1 have stored the partial sums of tile
+// `local` of a lattice observed at `step`. The block that completes a group of
+// OBS_GROUP tiles adds the group up, the one that completes the last group
+// adds the groups up and writes the record: in a fixed order, whichever block
+// it is. (Two launches after every step that recorded did this before: 5 us
+// per step of a small lattice.) red: NT / 32 * NOBS doubles, flag: one int of
+// shared memory, both written again only after a barrier.
+template <int NT, typename Sync>
+__device__ __forceinline__ void finish_obs(const LatDesc& d, int local, long long step, int tid, double* red, int* flag,
+                                           Sync sync) {
+    const int groups = (int)obs_groups(d.items), g = local / OBS_GROUP;
+    const int n = min(OBS_GROUP, d.items - g * OBS_GROUP);
+    auto last_of = [&](unsigned* count, int of) {
+        if (tid < NOBS) __threadfence();   // the sums these threads have stored
+        sync();
+        if (tid == 0) {
+            *flag = atomicAdd(count, 1u) == (unsigned)of - 1u;
+            __threadfence();
+        }
+        sync();
+        return *flag != 0;
+    };
+    if (!last_of(d.obs_count + g, n)) return;
+    sum_partials<NT>(d.partials + (long long)g * OBS_GROUP * NOBS, n, tid, red, sync);
+    if (tid == 0) d.obs_count[g] = 0;
+    if (groups > 1) {
+        if (tid < NOBS) {
+            double t = 0.0;
+            for (int w = 0; w < NT / 32; ++w) t += red[w * NOBS + tid];
+            d.group_partials[(long long)g * NOBS + tid] = t;
+        }
+        if (!last_of(d.obs_count + groups, groups)) return;
+        sum_partials<NT>(d.group_partials, groups, tid, red, sync);
+        if (tid == 0) d.obs_count[groups] = 0;
+    }
+    if (tid == 0) {
+        double tot[NOBS];
+        for (int q = 0; q < NOBS; ++q) {
+            tot[q] = 0.0;
+            for (int w = 0; w < NT / 32; ++w) tot[q] += red[w * NOBS + q];
+        }
+        d.series[(step - d.obs_base) / d.obs_every] =
+            make_obs(step, d.dt, d.nx, d.ny, d.rho0, d.probe_comp, d.probe_norm, tot);
+    }
 }
 
 }  // namespace lbm

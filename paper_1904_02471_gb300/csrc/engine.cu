@@ -131,7 +131,8 @@ Engine::~Engine() {
         cudaFree(g.d_item_begin);
         cudaFree(g.d_hdr);
         cudaFree(g.d_partials);
-        cudaFree(g.d_chunks);
+        cudaFree(g.d_group_partials);
+        cudaFree(g.d_obs_count);
     }
     if (own_stream_ && stream_) cudaStreamDestroy(stream_);
 }
@@ -382,16 +383,12 @@ int Engine::upload_group(int gi) {
     const int ty = g.model == LBM_CS ? cs_tile_ty(g.tile) : fd_tile_ty(g.tile);
     std::vector<int> begins;
     long long items = 0;
-    const bool had_obs = g.any_obs;
-    g.any_obs = false;
     for (int li : g.members) {
         const Lattice& L = lat[li];
         begins.push_back((int)items);
         items += (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty);
-        if (L.obs_every > 0) g.any_obs = true;
     }
     if (items >= (1LL << 31)) { set_error("too many work items"); return LBM_EINVAL; }
-    if (g.any_obs != had_obs) invalidate_graph();
     const int nm = (int)g.members.size();
     if (nm > g.cap_lat) {
         cudaFree(g.d_desc);
@@ -415,27 +412,31 @@ int Engine::upload_group(int gi) {
         g.cap_items = cap;
         invalidate_graph();
     }
-    g.total_items = (int)items;
-    long long max_items = 1;
-    for (int li : g.members) {
-        const Lattice& L = lat[li];
-        max_items = std::max<long long>(max_items, (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty));
-    }
-    // chunks of the observables reduction; fixed for dynamic engines so that
-    // membership changes do not change the captured launches
-    const int nch = dynamic_ ? 128 : (int)std::min<long long>(128, std::max<long long>(1, (max_items + 2047) / 2048));
-    if (nch != g.nchunks || (long long)g.cap_lat * nch > g.chunk_cap || !g.d_chunks) {
-        cudaFree(g.d_chunks);
-        g.d_chunks = nullptr;
-        g.nchunks = nch;
-        g.chunk_cap = g.cap_lat * nch;
-        CK(cudaMalloc(&g.d_chunks, sizeof(double) * NOBS * g.chunk_cap));
+    // group sums and counters of the observables: a lattice of n tiles has
+    // obs_groups(n) groups and one counter more
+    const long long slots = obs_groups(items) + 2LL * nm;
+    if (slots > g.cap_obs) {
+        cudaFree(g.d_group_partials);
+        cudaFree(g.d_obs_count);
+        g.d_group_partials = nullptr;
+        g.d_obs_count = nullptr;
+        const long long cap = std::max(slots, dynamic_ ? 2 * g.cap_obs : 0);
+        CK(cudaMalloc(&g.d_group_partials, sizeof(double) * NOBS * cap));
+        CK(cudaMalloc(&g.d_obs_count, sizeof(unsigned) * cap));
+        g.cap_obs = cap;
         invalidate_graph();
     }
+    if (nm) CK(cudaMemsetAsync(g.d_obs_count, 0, sizeof(unsigned) * g.cap_obs, stream_));
+    g.total_items = (int)items;
     std::vector<LatDesc> descs;
+    long long obs_slot = 0;
     for (int m = 0; m < nm; ++m) {
         lat[g.members[m]].slot = m;
-        descs.push_back(make_desc(lat[g.members[m]], g, begins[m], g.d_partials + (long long)begins[m] * NOBS));
+        LatDesc d = make_desc(lat[g.members[m]], g, begins[m], g.d_partials + (long long)begins[m] * NOBS);
+        d.group_partials = g.d_group_partials + obs_slot * NOBS;
+        d.obs_count = g.d_obs_count + obs_slot;
+        obs_slot += obs_groups(d.items) + 1;
+        descs.push_back(d);
     }
     const int hdr[4] = {nm, (int)items, 0, inject_us_};
     if (nm) {
@@ -489,21 +490,11 @@ int Engine::enqueue_chunk(int c) {
                 e = launch_cs_step(g.precision, g.tile, g.grid, gd, j, stream_);
                 if (e != cudaSuccess) return cuda_fail(e, "launch_cs_step");
                 ++n;
-                if (g.any_obs) {
-                    if ((e = launch_obs_finalize(gd, g.cap_lat, g.nchunks, g.d_chunks, j, stream_)) != cudaSuccess)
-                        return cuda_fail(e, "launch_obs_finalize");
-                    n += 2;
-                }
             } else {
                 for (int st = 1; st <= fd_stages(g.scheme); ++st) {
                     e = launch_fd_stage(g.precision, g.q1, g.scheme, g.tile, g.grid, gd, j, st, stream_);
                     if (e != cudaSuccess) return cuda_fail(e, "launch_fd_stage");
                     ++n;
-                    if (st == 1 && g.any_obs) {
-                        if ((e = launch_obs_finalize(gd, g.cap_lat, g.nchunks, g.d_chunks, j, stream_)) != cudaSuccess)
-                            return cuda_fail(e, "launch_obs_finalize");
-                        n += 2;
-                    }
                 }
             }
         }
@@ -608,16 +599,6 @@ int Engine::step_profiled(long long n, double* ms, int cap, double* total_ms) {
                 if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "profiled launch"); }
                 ++launches_;
                 marks.push_back({gi * 4 + (st - 1), a, b});
-                if (st == 1 && g.any_obs) {
-                    cudaEvent_t c = ev(), d = ev();
-                    if (!c || !d) { cleanup(); return cuda_fail(cudaGetLastError(), "cudaEventCreate"); }
-                    cudaEventRecord(c, stream_);
-                    e = launch_obs_finalize(gd, g.cap_lat, g.nchunks, g.d_chunks, 0, stream_);
-                    cudaEventRecord(d, stream_);
-                    if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "profiled finalize"); }
-                    launches_ += 2;
-                    marks.push_back({gi * 4 + 3, c, d});
-                }
             }
         }
         for (auto& g : groups) {

@@ -91,12 +91,10 @@ struct Group {
     int* d_hdr = nullptr;
     double* d_partials = nullptr;
     int cap_lat = 0;
-    long long cap_items = 0;
+    long long cap_items = 0, cap_obs = 0;
     int total_items = 0;
-    bool any_obs = false;
-    int nchunks = 1;            // observables reduction chunks per lattice
-    double* d_chunks = nullptr; // [cap_lat][nchunks][NOBS]
-    int chunk_cap = 0;
+    double* d_group_partials = nullptr;   // [sum of obs_groups][NOBS]
+    unsigned* d_obs_count = nullptr;      // [sum of obs_groups + 1]
     GroupDev dev() const { return GroupDev{d_desc, d_item_begin, d_hdr}; }
 };
 
@@ -129,7 +127,7 @@ class Engine {
     int step(long long n);
     // n steps launched one by one with CUDA events around every kernel;
     // ms[g * 4 + kind] accumulates the device time of group g's kernels of
-    // kind 0..2 (CS step, or FD stages 1..3) and 3 (observables finalise);
+    // kind 0..2 (CS step, or FD stages 1..3; kind 3 stays 0);
     // *total_ms spans the whole sequence.
     int step_profiled(long long n, double* ms, int cap, double* total_ms);
     long long kernel_launches() const { return launches_; }

@@ -50,10 +50,6 @@ int fd_blocks_per_sm(int precision, int q1, int tile, int scheme);
 // variants are refused by set_group_config and skipped by the autotuner.
 bool fd_variant_fits(int precision, int q1, int tile, int scheme);
 
-// Fused-observables finalisation: lattices observing at sub-step j reduce
-// their tile partials (in nchunks chunks, scratch chunks[max_lat][nchunks][NOBS])
-// into their series. Two launches.
-cudaError_t launch_obs_finalize(const GroupDev& g, int max_lat, int nchunks, double* chunks, int j, cudaStream_t s);
 // Advance steps/phase of every lattice by min(remaining, c).
 cudaError_t launch_advance(const GroupDev& g, int max_lat, int c, int flip_phase, cudaStream_t s);
 

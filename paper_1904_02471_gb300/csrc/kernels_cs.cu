@@ -111,6 +111,7 @@ __device__ __forceinline__ void cs_plain_aa_rows(const LatDesc* dp, T* buf, int 
 template <typename T, int TX, int RY>
 __global__ void __launch_bounds__(TX) cs_step_kernel(GroupDev g, int j) {
     __shared__ double red[(TX / 32) * NOBS];
+    __shared__ int s_last;
     const int n_lat = g.hdr[0];
     const int total = g.hdr[1];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
@@ -200,7 +201,11 @@ __global__ void __launch_bounds__(TX) cs_step_kernel(GroupDev g, int j) {
                 }
             }
         }
-        if (obs) block_reduce_obs<T, TX>(acc, dp->partials + (long long)local * NOBS, red);
+        if (obs) {
+            block_reduce_obs<T, TX, false>(acc, dp->partials + (long long)local * NOBS, red);
+            finish_obs<TX>(*dp, local, dp->step0 + j, threadIdx.x, red, &s_last, [] { __syncthreads(); });
+            __syncthreads();   // the next item writes red again
+        }
     }
 }
 
@@ -377,6 +382,7 @@ __global__ void __launch_bounds__(32 + W, cs_bulk_min_blocks<T, W>()) cs_bulk_ke
     uint64_t* full = reinterpret_cast<uint64_t*>(sm + (size_t)S * SLOT_BYTES);
     uint64_t* empty = full + S;
     double* red = reinterpret_cast<double*>(empty + S);
+    __shared__ int s_last;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -488,7 +494,8 @@ __global__ void __launch_bounds__(32 + W, cs_bulk_min_blocks<T, W>()) cs_bulk_ke
                 for (int w = 0; w < NCW; ++w) t += red[w * NOBS + ctid];
                 dp->partials[(long long)local * NOBS + ctid] = t;
             }
-            named_sync(1, W);
+            finish_obs<W>(*dp, local, dp->step0 + j, ctid, red, &s_last, [] { named_sync(1, W); });
+            named_sync(1, W);   // the next item writes red again
         }
     }
 }

@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     __shared__ unsigned char s_dead[LATS];
     __shared__ __align__(16) LatDesc s_desc[4];
     __shared__ int s_item[4];
+    __shared__ int s_last;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int grp = lane / LC, c0 = (lane % LC) * N;   // row group and first column of the lane's nodes
@@ -612,6 +613,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     for (int w = 0; w < NA; ++w) s += red[w * NOBS + atid];
                     cp->partials[(long long)local * NOBS + atid] = s;
                 }
+                finish_obs<NA * 32>(*cp, local, cp->step0 + j, atid, red, &s_last, [] { named_sync(1, NA * 32); });
             }
             named_arrive(2 + b, Ge::NT);
         }
@@ -690,9 +692,10 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             };
             // rows unrolled: all of them, or two where the copies for the signs
             // of v_x (three with an odd set) would outgrow the instruction cache
-            constexpr int UN = IMEX && Q1 == 4 ? HS : (Q1 == 3 && HS > 2 ? 2 : (Q1 == 5 && HS > 4 ? 2 : HS));
+            // (IMEX: or the registers)
+            constexpr int UN = IMEX || Q1 == 3 ? (HS < 2 ? HS : 2) : (Q1 == 5 && HS > 4 ? 2 : HS);
             // the node values are loaded AH rows ahead of their use
-            constexpr int AH = Q1 == 4 ? (IMEX ? (HS < 2 ? HS : 2) : HS) : UN;
+            constexpr int AH = Q1 == 4 && !IMEX ? HS : UN;
             V fq[AH];
             [[maybe_unused]] V pq[IMEX ? AH : 1];
 #pragma unroll

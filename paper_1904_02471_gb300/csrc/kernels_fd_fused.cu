@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
     double* red = reinterpret_cast<double*>(mom + Ge::n_m);
     __shared__ long long s_row[H0];            // wrapped row offsets of the staged rows
     __shared__ int s_col[W0];                  // wrapped columns of the staged columns
-    __shared__ int s_obs;
+    __shared__ int s_obs, s_last;
     __shared__ T s_vx[K], s_vy[K], s_w[K];
 
     const int n_lat = g.hdr[0];
@@ -331,7 +331,10 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
                 }
             }
             // no trailing barrier: `red` is next written after this item's barriers
-            if (s_obs) block_reduce_obs<T, NT, false>(acc, dp->partials + (long long)local * NOBS, red);
+            if (s_obs) {
+                block_reduce_obs<T, NT, false>(acc, dp->partials + (long long)local * NOBS, red);
+                finish_obs<NT>(*dp, local, dp->step0 + j, tid, red, &s_last, [] { __syncthreads(); });
+            }
         }
         for (int k0 = 0, gi = 0; k0 < K; k0 += G, ++gi) {
             const int ng = K - k0 < G ? K - k0 : G;

@@ -160,41 +160,6 @@ __global__ void __launch_bounds__(FIN_THREADS) snap_finalize_kernel(LatDesc* d, 
     if (threadIdx.x < NOBS) d->snap[threadIdx.x] = tot[threadIdx.x];
 }
 
-__device__ void write_record(LatDesc* d, long long step, const double* tot) {
-    d->series[(step - d->obs_base) / d->obs_every] =
-        make_obs(step, d->dt, d->nx, d->ny, d->rho0, d->probe_comp, d->probe_norm, tot);
-}
-
-// Two-level reduction of the tile partials of every lattice observing at
-// sub-step j: chunk sums (grid max_lat x nchunks), then one block per lattice
-// sums its chunks in order and writes the record.
-__global__ void __launch_bounds__(FIN_THREADS) obs_chunk_kernel(GroupDev g, int j, int nchunks, double* chunks) {
-    __shared__ double sm[FIN_THREADS * NOBS];
-    __shared__ double tot[NOBS];
-    const int li = blockIdx.x / nchunks, ch = blockIdx.x - li * nchunks;
-    if (li >= g.hdr[0]) return;
-    const LatDesc* d = g.desc + li;
-    if ((long long)j >= d->remaining || !observe_now(*d, j)) return;
-    const long long len = (d->items + nchunks - 1) / nchunks;
-    const long long lo = ch * len;
-    const long long hi = lo + len < d->items ? lo + len : d->items;
-    sum_rows(d->partials + lo * NOBS, hi > lo ? hi - lo : 0, tot, sm);
-    __syncthreads();
-    if (threadIdx.x < NOBS) chunks[((long long)li * nchunks + ch) * NOBS + threadIdx.x] = tot[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(FIN_THREADS) obs_finalize_kernel(GroupDev g, int j, int nchunks, const double* chunks) {
-    __shared__ double sm[FIN_THREADS * NOBS];
-    __shared__ double tot[NOBS];
-    const int li = blockIdx.x;
-    if (li >= g.hdr[0]) return;
-    LatDesc* d = g.desc + li;
-    if ((long long)j >= d->remaining || !observe_now(*d, j)) return;
-    sum_rows(chunks + (long long)li * nchunks * NOBS, nchunks, tot, sm);
-    __syncthreads();
-    if (threadIdx.x == 0) write_record(d, d->step0 + j, tot);
-}
-
 __global__ void advance_kernel(GroupDev g, int c, int flip) {
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
     if (li >= g.hdr[0]) return;
@@ -259,15 +224,6 @@ cudaError_t launch_readout(int precision, int q1, int pull, const LatDesc* d, in
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !part) return e;
     snap_finalize_kernel<<<1, FIN_THREADS, 0, s>>>(const_cast<LatDesc*>(d), part, grid);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_obs_finalize(const GroupDev& g, int max_lat, int nchunks, double* chunks, int j, cudaStream_t s) {
-    if (max_lat <= 0) return cudaSuccess;
-    obs_chunk_kernel<<<max_lat * nchunks, FIN_THREADS, 0, s>>>(g, j, nchunks, chunks);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    obs_finalize_kernel<<<max_lat, FIN_THREADS, 0, s>>>(g, j, nchunks, chunks);
     return cudaGetLastError();
 }
 

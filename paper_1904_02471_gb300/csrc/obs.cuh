@@ -84,19 +84,4 @@ __device__ __forceinline__ void sum_rows(const double* __restrict__ p, long long
     if (threadIdx.x < NOBS) out[threadIdx.x] = sm[threadIdx.x];
 }
 
-// The observables record of a state from its NOBS global sums.
-__device__ __forceinline__ lbm_obs make_obs(long long step, double dt, int nx, int ny, double rho0, int probe_comp,
-                                            double probe_norm, const double* tot) {
-    lbm_obs o;
-    o.step = step;
-    o.time = (double)step * dt;
-    o.mass = (double)nx * (double)ny * rho0 + tot[0];
-    o.mom_x = tot[1];
-    o.mom_y = tot[2];
-    o.amp = probe_comp >= 0 ? probe_norm * tot[3] : 0.0;
-    o.nonfinite = (isfinite(o.mass) && isfinite(o.amp) && isfinite(o.mom_x) && isfinite(o.mom_y)) ? 0 : 1;
-    o.reserved = 0;
-    return o;
-}
-
 }  // namespace lbm
