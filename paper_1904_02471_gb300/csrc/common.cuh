@@ -197,6 +197,27 @@ __device__ __forceinline__ bool observe_now(const LatDesc& d, int j) {
 }
 
 
+// 1 / x to within an ulp or two for a normal x far from the range limits:
+// the hardware's approximate reciprocal; double: refined by one third-order
+// Householder step r (1 + e + e^2), e = 1 - x r (three FP64 operations; the
+// FP64 pipe bounds the FP64 kernels, a division takes over twice as many).
+__device__ __forceinline__ float fast_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float fast_rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ double fast_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = ::fma(-x, r, 1.0);
+    return ::fma(::fma(e, e, e), r, r);
+}
+
 // Block reduction of NOBS per-thread partial sums into out[NOBS] (double).
 // Warp level in T (for FP32 storage: at most 32 per-thread sums in float),
 // across warps in double, fixed order (deterministic).
