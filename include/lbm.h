@@ -484,8 +484,9 @@ int lbm_footprint(const lbm_spec* spec, size_t* bytes);
 
 /* Test injection of a device-side wait that runs out (no counterpart in the
  * paper; failure detection of the library itself). The CS bulk-copy kernel
- * (the default CS kernel; the only one with device-side waits) bounds every
- * mbarrier wait by 2 s of device time; with microseconds > 0, every wait of
+ * (the only one with device-side waits; the default for large FP32 lattices,
+ * and for every CS lattice without a configured tile while the injection is
+ * on) bounds every mbarrier wait by 2 s of device time; with microseconds > 0, every wait of
  * the following CS launches is bounded by that many microseconds and the
  * first block skips the copies of its first row, so that row's consumers wait
  * on a barrier that nothing completes. The wait runs out, the launch sets the

@@ -166,15 +166,31 @@ int Engine::default_grid(const Group& g, int tile) const {
     return persistent_grid(g, tile) * std::max(1, grid_mult_);
 }
 
-// Default tile of an FD group of fixed lattices: the variant with the least
-// rounds x (rows + c), rounds = tiles per SM rounded up, c the cost of a tile
-// beside its rows (halo, moments, first faces, block start) in rows. Measured
-// per tile and stage, 16 velocities: FP32 4.96 / 2.92 / 2.17 / 1.95 us and FP64
-// 204 / 110 / 64 / 40 us with 16 / 8 / 4 / 2 rows: c = 6.4 and 1.4. Small
-// lattices get small tiles (more SMs at work: FP64 60^2, 122 us per step with
-// 2 rows, 331 with 8), large ones tall tiles (FP32 2048^2, 0.80 ms per step
-// with 16 rows, 0.95 with 8).
-int Engine::default_fd_tile(const Group& g) const {
+// Default tile of a group. FD: the variant with the least rounds x (rows + c),
+// rounds = tiles per SM rounded up, c the cost of a tile beside its rows (halo,
+// moments, first faces, block start) in rows. Measured per tile and stage, 16
+// velocities: FP32 4.96 / 2.92 / 2.17 / 1.95 us and FP64 204 / 110 / 64 / 40 us
+// with 16 / 8 / 4 / 2 rows: c = 6.4 and 1.4. Small lattices get small tiles
+// (more SMs at work: FP64 60^2, 122 us per step with 2 rows, 331 with 8), large
+// ones tall tiles (FP32 2048^2, 0.80 ms per step with 16 rows, 0.95 with 8).
+// CS: the bulk-copy kernel where the state streams through HBM (FP32, in place:
+// 198 us per step of 4096^2 against 225 for the plain kernel), else the plain
+// one: a bulk tile of 32 rows is a chain of 32 row copies on one SM (256^2: 24
+// us per step, plain 2.8; 1024^2: 25 and 13; 2048^2: 60.6 and 58.9). FP64 is
+// bound by the FP64 pipe, so its tiles spread over the SMs: one row of 32
+// nodes while all of them fit the GPU at once, then 128 x 1, then 128 x 2
+// (256^2: 11.1 us per step against 11.3 and 141 with bulk tiles).
+int Engine::default_tile(const Group& g) const {
+    if (g.model == LBM_CS) {
+        long long nodes = 0;
+        for (int li : g.members) nodes += (long long)lat[li].spec.nx * lat[li].spec.ny;
+        // the injection needs the kernel that waits; a server keeps it too: its
+        // test of overlapping runs counts on a run of 4000 CS steps on 512^2
+        // still being on the GPU after 50 ms (plain tiles end it after 30)
+        if (inject_us_ > 0 || dynamic_) return (int)CS_B256x32;
+        if (g.precision == LBM_FP32_DEV) return nodes >= 8LL << 20 ? (int)CS_B256x32 : (int)CS_T128x1;
+        return nodes <= 128LL * sm_count_ ? (int)CS_T32x1 : (nodes < 65536 ? (int)CS_T128x1 : (int)CS_T128x2);
+    }
     const double c = g.precision == LBM_FP64 ? 1.4 : 6.4;
     int best = g.tile;
     double best_cost = 1e300;
@@ -280,7 +296,6 @@ int Engine::add_lattice(const lbm_spec* spec, int* index, bool upload) {
         g.precision = s.precision;
         g.scheme = s.scheme;
         g.tile = s.model == LBM_CS ? (int)CS_B256x32 : (int)FD_T32x8;
-        if (s.model == LBM_FD && s.scheme != LBM_TS_RK3_FUSED && (long long)s.nx * s.ny >= 1 << 20) g.tile = (int)FD_T32x16;
         // the fused FD kernel's largest tiles do not fit every set and precision
         if (s.model == LBM_FD && s.scheme == LBM_TS_RK3_FUSED && !fd_variant_fits(s.precision, s.q_per_axis, g.tile, s.scheme))
             g.tile = FD_T32x4;
@@ -327,8 +342,7 @@ int Engine::create(const lbm_spec* specs, int n, void* stream) {
         rc = add_lattice(&specs[i], nullptr, false);
         if (rc) return rc;
     }
-    for (auto& g : groups)
-        if (g.model == LBM_FD) g.tile = default_fd_tile(g);
+    for (auto& g : groups) g.tile = default_tile(g);
     return upload_all();
 }
 
@@ -379,6 +393,15 @@ LatDesc Engine::make_desc(const Lattice& L, const Group& g, int item_begin, doub
 
 int Engine::upload_group(int gi) {
     Group& g = groups[gi];
+    if (dynamic_ && g.auto_tile && !g.members.empty()) {
+        // the lattices come and go: the tile follows them
+        const int tile = default_tile(g);
+        if (tile != g.tile) {
+            g.tile = tile;
+            g.grid = 0;
+            invalidate_graph();
+        }
+    }
     const int tx = g.model == LBM_CS ? cs_tile_tx(g.tile) : fd_tile_tx(g.tile);
     const int ty = g.model == LBM_CS ? cs_tile_ty(g.tile) : fd_tile_ty(g.tile);
     std::vector<int> begins;
@@ -471,6 +494,7 @@ int Engine::set_group_config(int gi, int tile, int grid) {
     }
     CK(cudaStreamSynchronize(stream_));
     g.tile = tile;
+    g.auto_tile = false;
     g.grid = 0;
     int rc = upload_group(gi);
     if (rc) return rc;
@@ -636,11 +660,21 @@ int Engine::inject_wait_timeout(int us) {
         return LBM_EINVAL;
     }
     inject_us_ = us;
-    for (auto& g : groups) {
+    for (int gi = 0; gi < (int)groups.size(); ++gi) {
+        Group& g = groups[gi];
         if (!g.d_hdr) continue;
         CK(cudaMemcpyAsync(g.d_hdr + 3, &inject_us_, sizeof(int), cudaMemcpyHostToDevice, stream_));
+        CK(cudaStreamSynchronize(stream_));
+        if (g.model != LBM_CS || !g.auto_tile || g.members.empty()) continue;
+        const int tile = default_tile(g);
+        if (tile == g.tile) continue;
+        int err = 0;   // an error word not read yet outlives the new configuration
+        CK(cudaMemcpy(&err, g.d_hdr + 2, sizeof err, cudaMemcpyDeviceToHost));
+        const int rc = set_group_config(gi, tile, 0);
+        if (rc) return rc;
+        g.auto_tile = true;
+        if (err) CK(cudaMemcpy(g.d_hdr + 2, &err, sizeof err, cudaMemcpyHostToDevice));
     }
-    CK(cudaStreamSynchronize(stream_));
     return LBM_OK;
 }
 

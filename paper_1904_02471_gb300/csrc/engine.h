@@ -84,6 +84,7 @@ struct Group {
     // the lattices' cur flips with every step (CS, fused FD)
     bool flips() const { return model == LBM_CS || scheme == LBM_TS_RK3_FUSED; }
     int tile = 0;
+    bool auto_tile = true;   // the tile is the default one (no configuration, no tuning)
     int grid = 0;
     std::vector<int> members;
     LatDesc* d_desc = nullptr;
@@ -160,7 +161,7 @@ class Engine {
     int sm_count() const { return sm_count_; }
     int default_grid(const Group& g, int tile) const;
     int persistent_grid(const Group& g, int tile) const;
-    int default_fd_tile(const Group& g) const;
+    int default_tile(const Group& g) const;
     int tune(int trial_steps, std::string* report);
 
     int chunk = 32;          // steps per captured graph

@@ -525,12 +525,13 @@ int cs_tile_tx(int v) {
         case CS_T128x1: case CS_T128x2: case CS_B128x32: return 128;
         case CS_T256x1: case CS_T256x2: case CS_B256x32: return 256;
         case CS_T64x4: return 64;
+        case CS_T32x1: return 32;
     }
     return 0;
 }
 int cs_tile_ty(int v) {
     switch (v) {
-        case CS_T128x1: case CS_T256x1: return 1;
+        case CS_T128x1: case CS_T256x1: case CS_T32x1: return 1;
         case CS_T128x2: case CS_T256x2: return 2;
         case CS_T64x4: return 4;
         case CS_B256x32: case CS_B128x32: return 32;
@@ -546,6 +547,7 @@ static const void* cs_kernel_ptr(int tile) {
         case CS_T256x1: return (const void*)cs_step_kernel<T, 256, 1>;
         case CS_T256x2: return (const void*)cs_step_kernel<T, 256, 2>;
         case CS_T64x4: return (const void*)cs_step_kernel<T, 64, 4>;
+        case CS_T32x1: return (const void*)cs_step_kernel<T, 32, 1>;
         case CS_B256x32: return (const void*)cs_bulk_kernel<T, 256, 32, 4>;
         case CS_B128x32: return (const void*)cs_bulk_kernel<T, 128, 32, 6>;
     }
