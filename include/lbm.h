@@ -342,8 +342,8 @@ int lbm_batch_groups(lbm_batch* b, int* model, int* q, int* precision, int cap);
 /* Measurement: n steps launched one kernel at a time with CUDA events around
  * every kernel (no graph). ms[g*4 + k] (cap entries, caller-owned) receives
  * the summed device time of group g's kernels of kind k: 0..2 = CS step or FD
- * stages 1..3 (entry 3 stays 0: observables are recorded inside those
- * kernels); *total_ms the span of all n steps. Computes exactly what lbm_batch_step(n) computes. Synchronous. */
+ * stages 1..3, 3 = observables finalisation where it is a launch of its own;
+ * *total_ms the span of all n steps. Computes exactly what lbm_batch_step(n) computes. Synchronous. */
 int lbm_batch_step_profiled(lbm_batch* b, int64_t n, double* ms, int cap, double* total_ms);
 
 /* Kernel configuration of group `group` of a batch (lbm_batch_groups order):

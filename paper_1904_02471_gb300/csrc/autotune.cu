@@ -47,7 +47,7 @@ int Engine::tune(int trial_steps, std::string* report) {
             std::lock_guard<std::mutex> lk(cache_mutex());
             auto it = cache().find(key);
             if (it != cache().end()) {
-                int rc = set_group_config(gi, it->second.first, 0);
+                int rc = apply_config(gi, it->second.first, 0);
                 if (rc) return rc;
                 g.grid = std::min(g.grid, std::max(1, it->second.second));
                 char b[160];
@@ -70,12 +70,12 @@ int Engine::tune(int trial_steps, std::string* report) {
             if (e != cudaSuccess) return cuda_fail(e, "tune save copy");
             saved.push_back(p);
         }
-        const int ntiles = g.model == LBM_CS ? (int)CS_NTILES : (int)FD_NTILES;
+        const int ntiles = g.model == LBM_CS ? (int)CS_NTILES : (int)FD_NALL;
         float best = 1e30f;
         int best_tile = g.tile, best_grid = g.grid;
         for (int t = 0; t < ntiles; ++t) {
             if (g.model == LBM_FD && !fd_variant_fits(g.precision, g.q1, t, g.scheme)) continue;
-            int rc = set_group_config(gi, t, 0);
+            int rc = apply_config(gi, t, 0);
             if (rc) return rc;
             const int full = g.total_items;
             const int pers = std::min(full, persistent_grid(g, t));
@@ -121,7 +121,7 @@ int Engine::tune(int trial_steps, std::string* report) {
         }
         cudaStreamSynchronize(stream_);
         for (void* p : saved) cudaFree(p);
-        int rc = set_group_config(gi, best_tile, best_grid);
+        int rc = apply_config(gi, best_tile, best_grid);
         if (rc) return rc;
         {
             std::lock_guard<std::mutex> lk(cache_mutex());

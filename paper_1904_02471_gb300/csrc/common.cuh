@@ -18,7 +18,7 @@
 
 namespace lbm {
 
-// Tiles whose partial sums one block adds up (finish_obs).
+// Rows of partial sums one block adds up (obs_add_group).
 constexpr int OBS_GROUP = 256;
 __host__ __device__ constexpr long long obs_groups(long long items) { return (items + OBS_GROUP - 1) / OBS_GROUP; }
 
@@ -51,9 +51,9 @@ struct alignas(16) LatDesc {   // copied in 16-byte chunks
     const double* probe_py;   // [ny]
     const float* probe_pxf;   // float copies for FP32 kernels
     const float* probe_pyf;
-    double* partials;       // [items][NOBS], this lattice's slice
-    double* group_partials; // [obs_groups][NOBS]: sums of OBS_GROUP tiles each
-    unsigned* obs_count;    // [obs_groups + 1]: tiles done of each group, groups done (0 between launches)
+    double* partials;       // [items][NOBS], this lattice's slice (rows of a launch's blocks)
+    double* group_partials; // [obs_groups][NOBS]: sums of OBS_GROUP rows each
+    unsigned* obs_count;    // [obs_groups + 1]: rows done of each group, groups done (0 between launches)
     lbm_obs* series;        // [obs_cap]
     double* snap;           // [NOBS] result of a one-off observables reduction
     // float copies of omega, cdx, dt_tau, rho0, eps for the FP32 kernels (a
@@ -287,39 +287,41 @@ __device__ __forceinline__ void sum_partials(const double* p, int n, int tid, do
     sync();
 }
 
-// Called by NT threads of a block (tid 0 .. NT - 1, `sync` a barrier of
-// theirs) after threads 0 .. NOBS - 1 have stored the partial sums of tile
-// `local` of a lattice observed at `step`. The block that completes a group of
-// OBS_GROUP tiles adds the group up, the one that completes the last group
-// adds the groups up and writes the record: in a fixed order, whichever block
-// it is. (Two launches after every step that recorded did this before: 5 us
-// per step of a small lattice.) red: NT / 32 * NOBS doubles, flag: one int of
-// shared memory, both written again only after a barrier.
+// The sums of a lattice observed at `step`, from rows of partial sums: block b
+// of a launch adds up the tiles it does (obs_tile below) and stores them as
+// row `its first tile of the lattice`; the first min(grid, items) tiles belong
+// to as many blocks, so those are the rows. All functions are called by NT
+// threads (tid 0 .. NT - 1, `sync` a barrier of theirs); red: NT / 32 * NOBS
+// doubles, flag: one int of shared memory.
+
+// Did this block count last of `of`? Its earlier stores (by threads below
+// NOBS) are visible to the block that does.
+template <typename Sync>
+__device__ __forceinline__ bool obs_last(unsigned* count, int of, int tid, int* flag, Sync sync) {
+    if (tid < NOBS) __threadfence();
+    sync();
+    if (tid == 0) {
+        *flag = atomicAdd(count, 1u) == (unsigned)of - 1u;
+        __threadfence();
+    }
+    sync();
+    return *flag != 0;
+}
+// Add up group g (OBS_GROUP rows) of the lattice's rows; the block that adds
+// up the last group adds the groups up and writes the record: in a fixed
+// order, whichever block it is.
 template <int NT, typename Sync>
-__device__ __forceinline__ void finish_obs(const LatDesc& d, int local, long long step, int tid, double* red, int* flag,
-                                           Sync sync) {
-    const int groups = (int)obs_groups(d.items), g = local / OBS_GROUP;
-    const int n = min(OBS_GROUP, d.items - g * OBS_GROUP);
-    auto last_of = [&](unsigned* count, int of) {
-        if (tid < NOBS) __threadfence();   // the sums these threads have stored
-        sync();
-        if (tid == 0) {
-            *flag = atomicAdd(count, 1u) == (unsigned)of - 1u;
-            __threadfence();
-        }
-        sync();
-        return *flag != 0;
-    };
-    if (!last_of(d.obs_count + g, n)) return;
-    sum_partials<NT>(d.partials + (long long)g * OBS_GROUP * NOBS, n, tid, red, sync);
-    if (tid == 0) d.obs_count[g] = 0;
+__device__ __forceinline__ void obs_add_group(const LatDesc& d, int g, int rows, long long step, int tid, double* red,
+                                              int* flag, Sync sync) {
+    const int groups = (int)obs_groups(rows);
+    sum_partials<NT>(d.partials + (long long)g * OBS_GROUP * NOBS, min(OBS_GROUP, rows - g * OBS_GROUP), tid, red, sync);
     if (groups > 1) {
         if (tid < NOBS) {
             double t = 0.0;
             for (int w = 0; w < NT / 32; ++w) t += red[w * NOBS + tid];
             d.group_partials[(long long)g * NOBS + tid] = t;
         }
-        if (!last_of(d.obs_count + groups, groups)) return;
+        if (!obs_last(d.obs_count + groups, groups, tid, flag, sync)) return;
         sum_partials<NT>(d.group_partials, groups, tid, red, sync);
         if (tid == 0) d.obs_count[groups] = 0;
     }
@@ -332,6 +334,42 @@ __device__ __forceinline__ void finish_obs(const LatDesc& d, int local, long lon
         d.series[(step - d.obs_base) / d.obs_every] =
             make_obs(step, d.dt, d.nx, d.ny, d.rho0, d.probe_comp, d.probe_norm, tot);
     }
+}
+// A block's tile `local` of an observed lattice: the threads' sums v are added
+// up (warp level in T: at most 32 per-thread sums in float; across warps and
+// tiles in double, in threads below NOBS) and the block's last tile of the
+// lattice stores its row. With `finish` the block that completes OBS_GROUP
+// rows goes on as above: no launch after the step (two such launches took 5 us
+// of every recorded step of a small lattice). Without it a launch of
+// obs_finish_kernel does: where a launch has thousands of blocks, a fence and
+// a count in each of them cost more (CS 8192^2: 0.767 ms per step against
+// 0.745).
+template <typename T, int NT, typename Sync>
+__device__ __forceinline__ void obs_tile(const T (&v)[NOBS], const LatDesc& d, int local, long long step, int tid,
+                                         double& run, double* red, int* flag, Sync sync, bool finish) {
+#pragma unroll
+    for (int q = 0; q < NOBS; ++q) {
+        T x = v[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((tid & 31) == 0) red[(tid >> 5) * NOBS + q] = (double)x;
+    }
+    sync();
+    const int grid = (int)gridDim.x;
+    if (tid < NOBS) {
+        double s = 0.0;
+        for (int w = 0; w < NT / 32; ++w) s += red[w * NOBS + tid];
+        run = local < grid ? s : run + s;
+    }
+    if (local + grid >= d.items) {
+        const int row = local % grid, rows = min(grid, d.items), g = row / OBS_GROUP;
+        if (tid < NOBS) d.partials[(long long)row * NOBS + tid] = run;
+        if (finish && obs_last(d.obs_count + g, min(OBS_GROUP, rows - g * OBS_GROUP), tid, flag, sync)) {
+            if (tid == 0) d.obs_count[g] = 0;
+            obs_add_group<NT>(d, g, rows, step, tid, red, flag, sync);
+        }
+    }
+    sync();   // red and flag are free again
 }
 
 }  // namespace lbm

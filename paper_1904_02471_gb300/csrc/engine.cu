@@ -128,11 +128,7 @@ Engine::~Engine() {
     for (auto& L : lat) free_lattice(L);
     for (auto& g : groups) {
         cudaFree(g.d_desc);
-        cudaFree(g.d_item_begin);
-        cudaFree(g.d_hdr);
         cudaFree(g.d_partials);
-        cudaFree(g.d_group_partials);
-        cudaFree(g.d_obs_count);
     }
     if (own_stream_ && stream_) cudaStreamDestroy(stream_);
 }
@@ -194,7 +190,7 @@ int Engine::default_tile(const Group& g) const {
     const double c = g.precision == LBM_FP64 ? 1.4 : 6.4;
     int best = g.tile;
     double best_cost = 1e300;
-    for (int t = 0; t < (int)FD_NTILES; ++t) {
+    for (int t = 0; t < (int)FD_NALL; ++t) {
         if (!fd_variant_fits(g.precision, g.q1, t, g.scheme)) continue;
         const int tx = fd_tile_tx(t), ty = fd_tile_ty(t);
         long long items = 0;
@@ -295,6 +291,7 @@ int Engine::add_lattice(const lbm_spec* spec, int* index, bool upload) {
         g.q1 = s.q_per_axis;
         g.precision = s.precision;
         g.scheme = s.scheme;
+        g.overlap = !dynamic_;
         g.tile = s.model == LBM_CS ? (int)CS_B256x32 : (int)FD_T32x8;
         // the fused FD kernel's largest tiles do not fit every set and precision
         if (s.model == LBM_FD && s.scheme == LBM_TS_RK3_FUSED && !fd_variant_fits(s.precision, s.q_per_axis, g.tile, s.scheme))
@@ -406,47 +403,43 @@ int Engine::upload_group(int gi) {
     const int ty = g.model == LBM_CS ? cs_tile_ty(g.tile) : fd_tile_ty(g.tile);
     std::vector<int> begins;
     long long items = 0;
+    g.min_every = 0;
     for (int li : g.members) {
         const Lattice& L = lat[li];
+        if (L.obs_every > 0) g.min_every = g.min_every > 0 ? std::min(g.min_every, L.obs_every) : L.obs_every;
         begins.push_back((int)items);
         items += (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty);
     }
     if (items >= (1LL << 31)) { set_error("too many work items"); return LBM_EINVAL; }
     const int nm = (int)g.members.size();
     if (nm > g.cap_lat) {
+        // one allocation: descriptors, the four header words, first items
         cudaFree(g.d_desc);
-        cudaFree(g.d_item_begin);
-        cudaFree(g.d_hdr);
         g.d_desc = nullptr;
         g.d_item_begin = nullptr;
         g.d_hdr = nullptr;
         const int cap = std::max(std::max(nm, 1), dynamic_ ? 2 * g.cap_lat : 0);  // grow geometrically
-        CK(cudaMalloc(&g.d_desc, sizeof(LatDesc) * cap));
-        CK(cudaMalloc(&g.d_item_begin, sizeof(int) * cap));
-        CK(cudaMalloc(&g.d_hdr, sizeof(int) * 4));
+        CK(cudaMalloc(&g.d_desc, sizeof(LatDesc) * cap + sizeof(int) * (4 + (size_t)cap)));
+        g.d_hdr = reinterpret_cast<int*>(g.d_desc + cap);
+        g.d_item_begin = g.d_hdr + 4;
         g.cap_lat = cap;
         invalidate_graph();
     }
-    if (items > g.cap_items) {
+    // one allocation: tile partials, group sums and counters of the observables
+    // (a lattice of n tiles has obs_groups(n) groups and one counter more)
+    const long long slots = obs_groups(items) + 2LL * nm;
+    if (items > g.cap_items || slots > g.cap_obs) {
         cudaFree(g.d_partials);
         g.d_partials = nullptr;
-        const long long cap = std::max(std::max<long long>(items, 1), dynamic_ ? 2 * g.cap_items : 0);
-        CK(cudaMalloc(&g.d_partials, sizeof(double) * NOBS * cap));
-        g.cap_items = cap;
-        invalidate_graph();
-    }
-    // group sums and counters of the observables: a lattice of n tiles has
-    // obs_groups(n) groups and one counter more
-    const long long slots = obs_groups(items) + 2LL * nm;
-    if (slots > g.cap_obs) {
-        cudaFree(g.d_group_partials);
-        cudaFree(g.d_obs_count);
         g.d_group_partials = nullptr;
         g.d_obs_count = nullptr;
-        const long long cap = std::max(slots, dynamic_ ? 2 * g.cap_obs : 0);
-        CK(cudaMalloc(&g.d_group_partials, sizeof(double) * NOBS * cap));
-        CK(cudaMalloc(&g.d_obs_count, sizeof(unsigned) * cap));
-        g.cap_obs = cap;
+        const long long ci = std::max(std::max<long long>(items, 1), dynamic_ ? 2 * g.cap_items : 0);
+        const long long co = std::max(slots, dynamic_ ? 2 * g.cap_obs : 0);
+        CK(cudaMalloc(&g.d_partials, sizeof(double) * NOBS * (ci + co) + sizeof(unsigned) * co));
+        g.d_group_partials = g.d_partials + ci * NOBS;
+        g.d_obs_count = reinterpret_cast<unsigned*>(g.d_group_partials + co * NOBS);
+        g.cap_items = ci;
+        g.cap_obs = co;
         invalidate_graph();
     }
     if (nm) CK(cudaMemsetAsync(g.d_obs_count, 0, sizeof(unsigned) * g.cap_obs, stream_));
@@ -492,6 +485,11 @@ int Engine::set_group_config(int gi, int tile, int grid) {
         set_error("this FD tile variant needs more shared memory than the device offers for this set/precision");
         return LBM_EINVAL;
     }
+    return apply_config(gi, tile, grid);
+}
+
+int Engine::apply_config(int gi, int tile, int grid) {
+    Group& g = groups[gi];
     CK(cudaStreamSynchronize(stream_));
     g.tile = tile;
     g.auto_tile = false;
@@ -503,6 +501,10 @@ int Engine::set_group_config(int gi, int tile, int grid) {
     return LBM_OK;
 }
 
+bool Engine::obs_launch(const Group& g) const {
+    return !g.finish_obs() && g.min_every > 0;
+}
+
 int Engine::enqueue_chunk(int c) {
     long long n = 0;
     for (int j = 0; j < c; ++j) {
@@ -510,15 +512,22 @@ int Engine::enqueue_chunk(int c) {
             if (g.cap_lat == 0) continue;  // empty groups launch too: kernels read the live count
             const GroupDev gd = g.dev();
             cudaError_t e;
+            auto finish = [&]() -> cudaError_t {
+                if (!obs_launch(g)) return cudaSuccess;
+                ++n;
+                return launch_obs_finish(gd, (int)g.members.size(), g.obs_rows(), g.grid, j, stream_);
+            };
             if (g.model == LBM_CS) {
                 e = launch_cs_step(g.precision, g.tile, g.grid, gd, j, stream_);
                 if (e != cudaSuccess) return cuda_fail(e, "launch_cs_step");
                 ++n;
+                if ((e = finish()) != cudaSuccess) return cuda_fail(e, "launch_obs_finish");
             } else {
                 for (int st = 1; st <= fd_stages(g.scheme); ++st) {
                     e = launch_fd_stage(g.precision, g.q1, g.scheme, g.tile, g.grid, gd, j, st, stream_);
                     if (e != cudaSuccess) return cuda_fail(e, "launch_fd_stage");
                     ++n;
+                    if (st == 1 && (e = finish()) != cudaSuccess) return cuda_fail(e, "launch_obs_finish");
                 }
             }
         }
@@ -623,6 +632,16 @@ int Engine::step_profiled(long long n, double* ms, int cap, double* total_ms) {
                 if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "profiled launch"); }
                 ++launches_;
                 marks.push_back({gi * 4 + (st - 1), a, b});
+                if (st == 1 && obs_launch(g)) {
+                    cudaEvent_t c = ev(), d = ev();
+                    if (!c || !d) { cleanup(); return cuda_fail(cudaGetLastError(), "cudaEventCreate"); }
+                    cudaEventRecord(c, stream_);
+                    e = launch_obs_finish(gd, (int)g.members.size(), g.obs_rows(), g.grid, 0, stream_);
+                    cudaEventRecord(d, stream_);
+                    if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "profiled finalize"); }
+                    ++launches_;
+                    marks.push_back({gi * 4 + 3, c, d});
+                }
             }
         }
         for (auto& g : groups) {

@@ -87,6 +87,8 @@ struct Group {
     bool auto_tile = true;   // the tile is the default one (no configuration, no tuning)
     int grid = 0;
     std::vector<int> members;
+    // two allocations, at d_desc (descriptors, header words, first items) and
+    // at d_partials (tile partials, group sums, counters)
     LatDesc* d_desc = nullptr;
     int* d_item_begin = nullptr;
     int* d_hdr = nullptr;
@@ -96,7 +98,18 @@ struct Group {
     int total_items = 0;
     double* d_group_partials = nullptr;   // [sum of obs_groups][NOBS]
     unsigned* d_obs_count = nullptr;      // [sum of obs_groups + 1]
-    GroupDev dev() const { return GroupDev{d_desc, d_item_begin, d_hdr}; }
+    bool overlap = true;        // launches may overlap (launch_overlapped)
+    // rows of partial sums of a launch (at most)
+    int obs_rows() const { return grid < total_items ? grid : total_items; }
+    // shortest recording interval of the members (0: none records)
+    long long min_every = 0;
+    // the step kernels finish the observables themselves, unless thousands of
+    // rows are recorded every few steps: a launch after every step then costs
+    // less than counting them (CS 8192^2, every step: 7 us against 22; CS
+    // 1000 x 777, every 20th: 0.8 us per step against nothing). A server's
+    // always do: its items change under a captured graph.
+    bool finish_obs() const { return !overlap || obs_rows() <= 4096 || min_every >= 4; }
+    GroupDev dev() const { return GroupDev{d_desc, d_item_begin, d_hdr, finish_obs() ? 1 : 0, overlap ? 1 : 0}; }
 };
 
 class Engine {
@@ -128,7 +141,7 @@ class Engine {
     int step(long long n);
     // n steps launched one by one with CUDA events around every kernel;
     // ms[g * 4 + kind] accumulates the device time of group g's kernels of
-    // kind 0..2 (CS step, or FD stages 1..3; kind 3 stays 0);
+    // kind 0..2 (CS step, or FD stages 1..3) and 3 (observables finalise);
     // *total_ms spans the whole sequence.
     int step_profiled(long long n, double* ms, int cap, double* total_ms);
     long long kernel_launches() const { return launches_; }
@@ -155,7 +168,8 @@ class Engine {
     int load(int i, const void* buf, size_t size);
 
     // Tile / grid selection for a group (autotuner hooks).
-    int set_group_config(int g, int tile, int grid);
+    int set_group_config(int g, int tile, int grid);   // public variants, checked
+    int apply_config(int g, int tile, int grid);
     int n_groups() const { return (int)groups.size(); }
     Group& G(int g) { return groups[g]; }
     int sm_count() const { return sm_count_; }
@@ -171,6 +185,8 @@ class Engine {
     int upload_group(int g);
     int upload_all();
     int enqueue_chunk(int c);
+    // the launch that finishes a step's observables, where one is needed
+    bool obs_launch(const Group& g) const;
     void mirror_advance(int c);
     int ensure_io(Lattice& L, size_t bytes);
     int readout(int i, double* f, double* rho, double* ux, double* uy, bool obs);

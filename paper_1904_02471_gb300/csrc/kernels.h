@@ -13,14 +13,39 @@ namespace lbm {
 struct GroupDev {
     LatDesc* desc;
     const int* item_begin;
-    int* hdr;   // {lattices, items, error bits, unused}
+    int* hdr;   // {lattices, items, error bits, wait-timeout injection}
+    int finish_obs;   // the step kernels finish the observables themselves (obs_tile)
+    int overlap;   // host side: launch_overlapped() may overlap this group's launches
 };
+
+// Launch of a kernel that starts with after_previous_launch(). With overlap its
+// blocks are placed while the previous launch on the stream drains, so that
+// the gap between two launches is no longer part of every step (25 velocities
+// on 2048 x 4: 15.7 -> 14.1 us per step; CS 1000 x 777: 13.4 -> 13.0). Not for
+// a server's two lanes: blocks that wait would hold SMs the other lane's
+// blocks could use (a mix of 10 runs: 50.4 -> 52.9 ms).
+inline cudaError_t launch_overlapped(const void* fn, int grid, int threads, void** args, size_t smem, cudaStream_t s,
+                                     bool overlap) {
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &a;
+    c.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelExC(&c, fn, args);
+}
 
 // Tile variants. CS: TX threads along x, RY rows per thread; the B
 // variants are the warp-specialised bulk-copy kernel (W columns x RB rows).
 // FD: TX x TY cells per tile, one cell per thread.
 enum CsTile { CS_T128x1 = 0, CS_T128x2, CS_T256x1, CS_T256x2, CS_T64x4, CS_B256x32, CS_B128x32, CS_T32x1, CS_NTILES };
-enum FdTile { FD_T32x8 = 0, FD_T32x4, FD_T32x16, FD_T32x2, FD_NTILES };
+// FD_T32x1 (FP64 stages only) is picked by the default rule and the tuner, not
+// by configuration.
+enum FdTile { FD_T32x8 = 0, FD_T32x4, FD_T32x16, FD_T32x2, FD_NTILES, FD_T32x1 = FD_NTILES, FD_NALL };
 
 int cs_tile_tx(int v);
 int cs_tile_ty(int v);
@@ -50,6 +75,9 @@ int fd_blocks_per_sm(int precision, int q1, int tile, int scheme);
 // variants are refused by set_group_config and skipped by the autotuner.
 bool fd_variant_fits(int precision, int q1, int tile, int scheme);
 
+// Observables of the lattices observed at sub-step j, after a step kernel
+// launched with `grid` blocks that did not finish them (finish_obs = 0).
+cudaError_t launch_obs_finish(const GroupDev& g, int lattices, int rows, int grid, int j, cudaStream_t s);
 // Advance steps/phase of every lattice by min(remaining, c).
 cudaError_t launch_advance(const GroupDev& g, int max_lat, int c, int flip_phase, cudaStream_t s);
 

@@ -175,8 +175,10 @@ template <typename T, int TX, int RY>
 __global__ void __launch_bounds__(TX) cs_step_kernel(GroupDev g, int j) {
     __shared__ double red[(TX / 32) * NOBS];
     __shared__ int s_last;
+    after_previous_launch();
     const int n_lat = g.hdr[0];
     const int total = g.hdr[1];
+    double run = 0.0;   // observables of this block's tiles so far
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int li = find_lattice(g.item_begin, n_lat, item);
         const LatDesc* dp = g.desc + li;
@@ -242,11 +244,9 @@ __global__ void __launch_bounds__(TX) cs_step_kernel(GroupDev g, int j) {
                 if (obs) cs_observe<T>(n, pc, pxv, dp, y, acc);
             }
         }
-        if (obs) {
-            block_reduce_obs<T, TX, false>(acc, dp->partials + (long long)local * NOBS, red);
-            finish_obs<TX>(*dp, local, dp->step0 + j, threadIdx.x, red, &s_last, [] { __syncthreads(); });
-            __syncthreads();   // the next item writes red again
-        }
+        if (obs)
+            obs_tile<T, TX>(acc, *dp, local, dp->step0 + j, threadIdx.x, run, red, &s_last, [] { __syncthreads(); },
+                            g.finish_obs != 0);
     }
 }
 
@@ -413,6 +413,7 @@ __global__ void __launch_bounds__(32 + W, cs_bulk_min_blocks<T, W>()) cs_bulk_ke
         fence_mbar_init();
     }
     __syncthreads();
+    after_previous_launch();
     const int n_lat = g.hdr[0];
     const int total = g.hdr[1];
     const int inject_us = g.hdr[3];
@@ -461,6 +462,7 @@ __global__ void __launch_bounds__(32 + W, cs_bulk_min_blocks<T, W>()) cs_bulk_ke
     const int ctid = threadIdx.x - 32;
     unsigned it = 0;
     bool dead = false;
+    double run = 0.0;   // observables of this block's tiles so far
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int li = find_lattice(g.item_begin, n_lat, item);
         const LatDesc* dp = g.desc + li;
@@ -496,27 +498,9 @@ __global__ void __launch_bounds__(32 + W, cs_bulk_min_blocks<T, W>()) cs_bulk_ke
         else
             cs_bulk_consume<T, W, S, CS_AA_ODD>(ring, full, empty, in, out, dp, x0, y0, y1, omega, r0, obs, pxv, it,
                                                 dead, g.hdr + 2, lim, acc);
-        if (obs) {
-            T r[NOBS];
-#pragma unroll
-            for (int q = 0; q < NOBS; ++q) {
-                T v = acc[q];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                r[q] = v;
-            }
-            if (lane == 0)
-#pragma unroll
-                for (int q = 0; q < NOBS; ++q) red[(warp - 1) * NOBS + q] = (double)r[q];
-            named_sync(1, W);
-            if (ctid < NOBS) {
-                double t = 0.0;
-                for (int w = 0; w < NCW; ++w) t += red[w * NOBS + ctid];
-                dp->partials[(long long)local * NOBS + ctid] = t;
-            }
-            finish_obs<W>(*dp, local, dp->step0 + j, ctid, red, &s_last, [] { named_sync(1, W); });
-            named_sync(1, W);   // the next item writes red again
-        }
+        if (obs)
+            obs_tile<T, W>(acc, *dp, local, dp->step0 + j, ctid, run, red, &s_last, [] { named_sync(1, W); },
+                           g.finish_obs != 0);
     }
 }
 
@@ -593,7 +577,7 @@ cudaError_t launch_cs_step(int precision, int tile, int grid, const GroupDev& g,
     GroupDev gg = g;
     int jj = j;
     void* args[] = {&gg, &jj};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(cs_threads(tile)), args, cs_bytes(precision, tile), s);
+    return launch_overlapped(fn, grid, cs_threads(tile), args, cs_bytes(precision, tile), s, g.overlap != 0);
 }
 
 int cs_blocks_per_sm(int precision, int tile) {

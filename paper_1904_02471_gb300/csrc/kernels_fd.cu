@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     const int grp = lane / LC, c0 = (lane % LC) * N;   // row group and first column of the lane's nodes
     constexpr int DCH = sizeof(LatDesc) / 16;          // 16-byte chunks of a descriptor
     static_assert(sizeof(LatDesc) % 16 == 0 && DCH <= 32, "descriptors are copied in 16-byte chunks by one warp");
+    after_previous_launch();
     // a lone lattice's descriptor is read while the group's header is on its way
     if (tid < DCH) reinterpret_cast<uint4*>(s_desc)[tid] = reinterpret_cast<const uint4*>(g.desc)[tid];
     const int n_lat = g.hdr[0];
@@ -416,6 +417,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
         if (aw == 0) look_up(blockIdx.x, 0);
         cp_async_wait_all();
         named_sync(1, NA * 32);
+        double run = 0.0;   // observables of this block's tiles so far
         for (unsigned n = 0;; ++n) {
             const int slot = n & 3;
             const int b = NB == 2 ? n & 1 : 0;
@@ -598,23 +600,9 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     }
                 }
             }
-            if (obs) {
-                // fixed order: lanes, then warps
-#pragma unroll
-                for (int q = 0; q < NOBS; ++q) {
-                    T v = acc[q];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane == 0) red[aw * NOBS + q] = (double)v;
-                }
-                named_sync(1, NA * 32);
-                if (atid < NOBS) {
-                    double s = 0.0;
-                    for (int w = 0; w < NA; ++w) s += red[w * NOBS + atid];
-                    cp->partials[(long long)local * NOBS + atid] = s;
-                }
-                finish_obs<NA * 32>(*cp, local, cp->step0 + j, atid, red, &s_last, [] { named_sync(1, NA * 32); });
-            }
+            if (obs)
+                obs_tile<T, NA * 32>(acc, *cp, local, cp->step0 + j, atid, run, red, &s_last,
+                                     [] { named_sync(1, NA * 32); }, g.finish_obs != 0);
             named_arrive(2 + b, Ge::NT);
         }
         return;
@@ -799,13 +787,14 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     }
 }
 
-int fd_tile_tx(int v) { return (v >= 0 && v < FD_NTILES) ? FD_TX : 0; }
+int fd_tile_tx(int v) { return (v >= 0 && v < FD_NALL) ? FD_TX : 0; }
 int fd_tile_ty(int v) {
     switch (v) {
         case FD_T32x8: return 8;
         case FD_T32x4: return 4;
         case FD_T32x16: return 16;
         case FD_T32x2: return 2;
+        case FD_T32x1: return 1;
     }
     return 0;
 }
@@ -830,6 +819,8 @@ static FdVariant fd_variant_q(int tile) {
         case FD_T32x4: return fd_variant_of<T, Q1, 4, IMEX>();
         case FD_T32x16: return fd_variant_of<T, Q1, 16, IMEX>();
         case FD_T32x2: return fd_variant_of<T, Q1, 2, IMEX>();
+        case FD_T32x1:
+            if constexpr (sizeof(T) == 8) return fd_variant_of<T, Q1, 1, IMEX>();
     }
     return FdVariant{};
 }
@@ -854,7 +845,7 @@ static FdVariant fd_variant(int precision, int tile, int q1, int scheme) {
 static cudaError_t fd_prepare(int precision, int tile, int q1) {
     // 0 unknown, 1 ready, 2 does not fit; atomic: the two lanes of a server
     // may prepare the same variant at once (both then make the same calls)
-    static std::atomic<int> state[2][FD_NTILES][3] = {};
+    static std::atomic<int> state[2][FD_NALL][3] = {};
     const int p = precision == LBM_FP64 ? 0 : 1;
     std::atomic<int>& st = state[p][tile][q1 - 3];
     if (st == 1) return cudaSuccess;
@@ -868,7 +859,7 @@ static cudaError_t fd_prepare(int precision, int tile, int q1) {
     for (int scheme : {LBM_TS_RK3, LBM_TS_IMEX}) {
         const FdVariant v = fd_variant(precision, tile, q1, scheme);
         cudaFuncAttributes a;
-        if (v.bytes > (size_t)optin || cudaFuncGetAttributes(&a, v.fn) != cudaSuccess ||
+        if (!v.fn || v.bytes > (size_t)optin || cudaFuncGetAttributes(&a, v.fn) != cudaSuccess ||
             // the shares must not exceed the registers the block is launched
             // with (a warpgroup would wait for the rest for ever)
             v.regs > (a.numRegs + 7) / 8 * 8 * v.threads ||
@@ -884,7 +875,7 @@ static cudaError_t fd_prepare(int precision, int tile, int q1) {
 
 cudaError_t launch_fd_stage(int precision, int q1, int scheme, int tile, int grid, const GroupDev& g, int j,
                             int stage, cudaStream_t s) {
-    if (tile < 0 || tile >= FD_NTILES || grid <= 0 || q1 < 3 || q1 > 5 ||
+    if (tile < 0 || tile >= FD_NALL || grid <= 0 || q1 < 3 || q1 > 5 ||
         (scheme != LBM_TS_RK3 && scheme != LBM_TS_IMEX && scheme != LBM_TS_RK3_FUSED) || stage < 1 ||
         stage > fd_stages(scheme))
         return cudaErrorInvalidValue;
@@ -895,12 +886,12 @@ cudaError_t launch_fd_stage(int precision, int q1, int scheme, int tile, int gri
     GroupDev gg = g;
     int jj = j, ss = stage;
     void* args[] = {&gg, &jj, &ss};
-    return cudaLaunchKernel(v.fn, dim3(grid), dim3(v.threads), args, v.bytes, s);
+    return launch_overlapped(v.fn, grid, v.threads, args, v.bytes, s, g.overlap != 0);
 }
 
 bool fd_variant_fits(int precision, int q1, int tile, int scheme) {
     if (scheme == LBM_TS_RK3_FUSED) return fd_fused_fits(precision, q1, tile);
-    return tile >= 0 && tile < FD_NTILES && q1 >= 3 && q1 <= 5 && fd_prepare(precision, tile, q1) == cudaSuccess;
+    return tile >= 0 && tile < FD_NALL && q1 >= 3 && q1 <= 5 && fd_prepare(precision, tile, q1) == cudaSuccess;
 }
 
 int fd_blocks_per_sm(int precision, int q1, int tile, int scheme) {

@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
     __shared__ int s_obs, s_last;
     __shared__ T s_vx[K], s_vy[K], s_w[K];
 
+    after_previous_launch();
     const int n_lat = g.hdr[0];
     const int total = g.hdr[1];
     const int tid = threadIdx.x;
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
         s_w[tid] = (T)w_of<Q1>(tid);
     }
 
+    double run = 0.0;   // observables of this block's tiles so far
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int li = find_lattice(g.item_begin, n_lat, item);
         const LatDesc* dp = g.desc + li;
@@ -330,11 +332,9 @@ __global__ void __launch_bounds__(FusedGeo<T, Q1, TY>::NT, 1) fd_fused_kernel(Gr
                     }
                 }
             }
-            // no trailing barrier: `red` is next written after this item's barriers
-            if (s_obs) {
-                block_reduce_obs<T, NT, false>(acc, dp->partials + (long long)local * NOBS, red);
-                finish_obs<NT>(*dp, local, dp->step0 + j, tid, red, &s_last, [] { __syncthreads(); });
-            }
+            if (s_obs)
+                obs_tile<T, NT>(acc, *dp, local, dp->step0 + j, tid, run, red, &s_last, [] { __syncthreads(); },
+                                g.finish_obs != 0);
         }
         for (int k0 = 0, gi = 0; k0 < K; k0 += G, ++gi) {
             const int ng = K - k0 < G ? K - k0 : G;
@@ -547,7 +547,7 @@ cudaError_t launch_fd_fused(int precision, int q1, int tile, int grid, const Gro
     GroupDev gg = g;
     int jj = j;
     void* args[] = {&gg, &jj};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(fd_fused_threads(precision)), args, bytes, s);
+    return launch_overlapped(fn, grid, fd_fused_threads(precision), args, bytes, s, g.overlap != 0);
 }
 
 }  // namespace lbm

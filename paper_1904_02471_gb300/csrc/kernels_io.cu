@@ -13,6 +13,7 @@
 // order by a single block (deterministic).
 #include "kernels.h"
 #include "obs.cuh"
+#include "ptx.cuh"
 
 namespace lbm {
 
@@ -160,7 +161,22 @@ __global__ void __launch_bounds__(FIN_THREADS) snap_finalize_kernel(LatDesc* d, 
     if (threadIdx.x < NOBS) d->snap[threadIdx.x] = tot[threadIdx.x];
 }
 
+// One block per lattice and group of OBS_GROUP rows (obs_add_group).
+__global__ void __launch_bounds__(FIN_THREADS) obs_finish_kernel(GroupDev g, int j, int grid, int groups) {
+    __shared__ double red[FIN_THREADS / 32 * NOBS];
+    __shared__ int s_last;
+    after_previous_launch();
+    const int li = blockIdx.x / groups, gr = blockIdx.x - li * groups;
+    if (li >= g.hdr[0]) return;
+    const LatDesc& d = g.desc[li];
+    if ((long long)j >= d.remaining || !observe_now(d, j)) return;
+    const int rows = min(grid, d.items);
+    if (gr >= obs_groups(rows)) return;
+    obs_add_group<FIN_THREADS>(d, gr, rows, d.step0 + j, threadIdx.x, red, &s_last, [] { __syncthreads(); });
+}
+
 __global__ void advance_kernel(GroupDev g, int c, int flip) {
+    after_previous_launch();
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
     if (li >= g.hdr[0]) return;
     LatDesc* d = g.desc + li;
@@ -227,10 +243,18 @@ cudaError_t launch_readout(int precision, int q1, int pull, const LatDesc* d, in
     return cudaGetLastError();
 }
 
+cudaError_t launch_obs_finish(const GroupDev& g, int lattices, int rows, int grid, int j, cudaStream_t s) {
+    GroupDev gg = g;
+    int groups = (int)obs_groups(rows);
+    void* args[] = {&gg, &j, &grid, &groups};
+    return launch_overlapped((const void*)obs_finish_kernel, lattices * groups, FIN_THREADS, args, 0, s, g.overlap != 0);
+}
+
 cudaError_t launch_advance(const GroupDev& g, int max_lat, int c, int flip_phase, cudaStream_t s) {
     if (max_lat <= 0) return cudaSuccess;
-    advance_kernel<<<(max_lat + 127) / 128, 128, 0, s>>>(g, c, flip_phase);
-    return cudaGetLastError();
+    GroupDev gg = g;
+    void* args[] = {&gg, &c, &flip_phase};
+    return launch_overlapped((const void*)advance_kernel, (max_lat + 127) / 128, 128, args, 0, s, g.overlap != 0);
 }
 
 }  // namespace lbm

@@ -107,6 +107,14 @@ __device__ __forceinline__ void named_arrive(int id, int nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Programmatic dependent launch. A step kernel's blocks may be on the SMs
+// before the launch they depend on has finished: every thread waits for it (and
+// for its writes) first, then lets the next launch come.
+__device__ __forceinline__ void after_previous_launch() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Change the registers per thread of the calling warpgroup (four aligned
 // warps, all of them executing it) within those the block was launched with.
 template <int N>
