@@ -844,8 +844,8 @@ def run_profile_case(a):
     Compute): a Taylor-Green lattice in FP32 deviation storage whose state is
     larger than the 129 MB L2 (CS 2048^2: 302 MB; FD 16-velocity 1024^2:
     201 MB) but small enough that a multi-pass capture ends in seconds. The
-    kernel variant can be pinned with --tile, the grid with --grid (0: one
-    block per tile)."""
+    kernel variant can be pinned with --tile, the grid with --grid (0: the
+    default)."""
     import torch
     import paper_1904_02471_gb300 as pkg
     torch.cuda.init()
@@ -891,7 +891,7 @@ def main():
     ap.add_argument("--n", type=int, default=0, help="--profile-case: lattice side")
     ap.add_argument("--case-steps", type=int, default=0, help="--profile-case: steps")
     ap.add_argument("--tile", type=int, default=-1, help="--profile-case: kernel tile variant")
-    ap.add_argument("--grid", type=int, default=0, help="--profile-case: grid (0: one block per tile)")
+    ap.add_argument("--grid", type=int, default=0, help="--profile-case: grid (0: the default, one block per tile for CS and at most one per SM for FD stages)")
     ap.add_argument("--q", type=int, default=4, help="--profile-case fd: nodes per axis")
     ap.add_argument("--precision", default="fp32", help="--profile-case: fp32 or fp64")
     ap.add_argument("--storage", default="ab", choices=["ab", "inplace"], help="--profile-case cs: storage")

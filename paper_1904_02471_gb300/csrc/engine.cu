@@ -167,7 +167,7 @@ int Engine::default_grid(const Group& g, int tile) const {
 // moments, first faces, block start) in rows. Measured per tile and stage, 16
 // velocities: FP32 4.96 / 2.92 / 2.17 / 1.95 us and FP64 204 / 110 / 64 / 40 us
 // with 16 / 8 / 4 / 2 rows: c = 6.4 and 1.4. Small lattices get small tiles
-// (more SMs at work: FP64 60^2, 122 us per step with 2 rows, 331 with 8), large
+// (more SMs at work: FP64 60^2, 35 us per step with 1 row, 48 with 2), large
 // ones tall tiles (FP32 2048^2, 0.80 ms per step with 16 rows, 0.95 with 8).
 // CS: the bulk-copy kernel where the state streams through HBM (FP32, in place:
 // 198 us per step of 4096^2 against 225 for the plain kernel), else the plain
