@@ -39,7 +39,6 @@ struct Pr<float> {
         return make_float2(__fmaf_rn(a.x, c, b.x), __fmaf_rn(a.y, c, b.y));
     }
     static __device__ __forceinline__ V rcp(V b) { return make_float2(fast_rcp(b.x), fast_rcp(b.y)); }
-    static __device__ __forceinline__ V rsqrt(V b) { return make_float2(fast_rsqrt(b.x), fast_rsqrt(b.y)); }
 };
 
 template <>

@@ -68,11 +68,11 @@ __device__ __forceinline__ void set_moments(Fn g, typename Lanes<T>::V& m0, type
     }
 }
 
-// The equilibrium at a node as five numbers (px, py, jx, jy, e0):
-//   stored f^eq_k = w_k (q_k + v_k . j + e0), i.e. Eq. (herfeq) minus w_k rho0.
-// FP32: p = j / sqrt(2 rho), q_k = (v_k . p)^2 = rho/2 (v_k . u)^2, e0 = dr - p^2;
-// FP64: p = u/2, q_k = (v_k . p)(v_k . j), e0 = dr - j . p (a square root
-// would cost more on the FP64 pipe than it saves).
+// The equilibrium at a node as five numbers, p = u / 2, j = rho u and e0 =
+// dr - j . p: stored f^eq_k / w_k = (v_k . p)(v_k . j) + v_k . j + e0, i.e. Eq.
+// (herfeq) minus w_k rho0. FP32 takes (1 + v_k . p)(v_k . j) + e0: five
+// operations, as many as the square of one product with p = j / sqrt(2 rho)
+// takes, and like Eq. (herfeq) defined for every density but zero.
 template <typename T>
 struct Equil {
     using P = Lanes<T>;
@@ -81,25 +81,18 @@ struct Equil {
     __device__ __forceinline__ void set(V rho, V dr, V jx_, V jy_) {
         jx = jx_;
         jy = jy_;
-        if constexpr (sizeof(T) == 4) {
-            const V s = P::rsqrt(P::add(rho, rho));
-            px = P::mul(jx, s);
-            py = P::mul(jy, s);
-            e0 = P::fma(P::neg(py), py, P::fma(P::neg(px), px, dr));
-        } else {
-            const V h = P::mulc(P::rcp(rho), T(0.5));
-            px = P::mul(jx, h);
-            py = P::mul(jy, h);
-            e0 = P::fma(-jy, py, P::fma(-jx, px, dr));
-        }
+        const V h = P::mulc(P::rcp(rho), T(0.5));
+        px = P::mul(jx, h);
+        py = P::mul(jy, h);
+        e0 = P::fma(P::neg(jy), py, P::fma(P::neg(jx), px, dr));
     }
     // (f^eq_k) / w_k; vx, vy: the population's velocity, broadcast
     __device__ __forceinline__ V over_w(V vx, V vy) const {
-        const V xi = P::fma(vx, px, P::mul(vy, py));
+        const V xj = P::fma(vx, jx, P::mul(vy, jy));
         if constexpr (sizeof(T) == 4) {
-            return P::fma(xi, xi, P::fma(vx, jx, P::fma(vy, jy, e0)));
+            return P::fma(P::fma(vx, px, P::fma(vy, py, P::sp(T(1)))), xj, e0);
         } else {
-            const V xj = P::fma(vx, jx, P::mul(vy, jy));
+            const V xi = P::fma(vx, px, P::mul(vy, py));
             return P::add(P::fma(xi, xj, xj), e0);
         }
     }
@@ -119,8 +112,8 @@ struct EquilAll {
 #pragma unroll
         for (int i = 0; i < Q1; ++i) {
             const T v = (T)GH<Q1>::v(i);
-            yp[i] = P::mulc(e.py, v);
-            yj[i] = sizeof(T) == 4 ? P::fmac(e.jy, v, e.e0) : P::mulc(e.jy, v);
+            yp[i] = sizeof(T) == 4 ? P::fmac(e.py, v, P::sp(T(1))) : P::mulc(e.py, v);
+            yj[i] = P::mulc(e.jy, v);
         }
     }
     // f^eq_k / w_k
@@ -128,7 +121,7 @@ struct EquilAll {
         const int ix = k % Q1, iy = k / Q1;
         const T v = (T)GH<Q1>::v(ix);
         const V xi = P::fmac(px, v, yp[iy]), vj = P::fmac(jx, v, yj[iy]);
-        if constexpr (sizeof(T) == 4) return P::fma(xi, xi, vj);
+        if constexpr (sizeof(T) == 4) return P::fma(xi, vj, e0);
         else return P::add(P::fma(xi, vj, vj), e0);
     }
 };
@@ -557,8 +550,9 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     // the viscous decay per stage of a slowly decaying flow. It is
                     // computed from the differences u_k - geq_k (accurate) and
                     // removed with w_k (R0 + v_k . R1), which has exactly these
-                    // moments (quadrature identities of the set): the linear part
-                    // of the equilibrium takes the shifted moments dr + R0, j + R1.
+                    // moments (quadrature identities of the set): the equilibrium
+                    // takes the shifted moments dr + R0, j + R1 (p . R1, which the
+                    // shifted j adds to its zeroth moment, is taken off e0).
                     if constexpr (sizeof(T) == 4) {
                         const T* U = static_cast<const T*>(cp->buf[in_idx]) + ((long long)(y0 + r) * pitch + x0 + c0);
                         const bool in = y0 + r < ny && x0 + c0 < nx;
@@ -576,7 +570,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                                 return P::fmac(ew, -(T)w_of<Q1>(k), u);
                             },
                             R0, R1x, R1y);
-                        e.e0 = P::add(e.e0, R0);
+                        e.e0 = P::add(e.e0, P::fma(P::neg(e.py), R1y, P::fma(P::neg(e.px), R1x, R0)));
                         e.jx = P::add(e.jx, R1x);
                         e.jy = P::add(e.jy, R1y);
                     }

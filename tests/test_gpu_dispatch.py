@@ -162,3 +162,23 @@ def test_recorded_sums_equal_the_snapshot(model, q, nx, ny, tile, scheme, prec):
         assert abs(s["mom_x"] - o["mom_x"]) <= eps * max(mu, full) and abs(s["mom_y"] - o["mom_y"]) <= eps * max(mv, full)
         assert abs(s["amp"] - o["amp"]) <= eps * max(mw, 1e-3 * full)
         assert s["nonfinite"] == 0
+
+
+@pytest.mark.parametrize("scheme", ["rk3", "imex", "rk3_fused"])
+@pytest.mark.parametrize("q", [3, 4, 5])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_fd_equilibrium_of_negative_density(q, scheme, prec):
+    """Eq. (herfeq) is odd in f: -f is a state like f, and its run is the run of
+    f with the sign changed. FP32 stores float32(f - w rho0), here of size
+    2 w: one rounding of 2^-24 of that per stage (12 of them) and in each
+    equilibrium and flux, amplified by less than 10 over four steps."""
+    nx, ny = 45, 22
+    f0 = _state(q, nx, ny, 13)
+    with _fd(q, nx, ny, scheme, prec) as L:
+        s = L.spec
+        L.set_populations(-f0)
+        L.step(4)
+        got = L.populations()
+    run = oracle.fd_imex_run if scheme == "imex" else oracle.fd_run
+    ref = run(-f0, s.dx, s.dt, s.tau, 4)
+    assert rel_err(got, ref) < (TOL64 if prec == "fp64" else 12 * 2 * 10 * 2.0 ** -24)
