@@ -430,41 +430,55 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             const int nx = cp->nx, ny = cp->ny, pitch = cp->pitch;
             const long long plane = cp->plane;
             // 1. the K halo tiles of the stage input: 16-byte asynchronous
-            //    copies (interior rows are 16-byte aligned: x0 - 4 is a multiple
-            //    of 4, the pitch of 32; at the periodic edge no chunk straddles
-            //    the wrap point when nx is a multiple of VEC), else single
-            //    values. A lane copies the same chunks of every population's
-            //    tile: their offsets are formed once per item (below 2^32: a
-            //    plane's elements times the three buffers fit the device).
+            //    copies (rows are 16-byte aligned: x0 - 4 is a multiple of 4, the
+            //    pitch of 32). At the periodic edge a chunk wraps as a whole when
+            //    nx is a multiple of VEC; otherwise the chunks before x = 0 and
+            //    across nx go value by value, and those no node of the lattice
+            //    reaches (beyond nx + 2) are left out (whole edge tiles value by
+            //    value: FD 16-velocity 777 x 500 took 1.4x the time). A lane
+            //    copies the same chunks of every population's tile: their offsets
+            //    are formed once per item (below 2^32: a plane's elements times
+            //    the three buffers fit the device).
             const T* const U0 = static_cast<const T*>(cp->buf[in_idx]);
             const bool interior = x0 >= 4 && x0 + TX + 4 <= nx && y0 >= 3 && y0 + TY + 3 <= ny;
-            if (interior || nx % VEC == 0) {
-                unsigned so[NIT];
+            unsigned so[NIT], whole = 0, part = 0;   // one bit per chunk of the lane
+#pragma unroll
+            for (int i = 0; i < NIT; ++i) {
+                const int q = lane + 32 * i, r = q / CH, c = (q - r * CH) * VEC;
+                const int y = y0 - 3 + r, x = x0 - 4 + c;
+                if ((i + 1) * 32 <= RT * CH || q < RT * CH) {
+                    if (interior || nx % VEC == 0 || (x >= 0 && x + VEC <= nx)) whole |= 1u << i;
+                    else if (x < nx + 3) part |= 1u << i;
+                }
+                so[i] = interior ? (unsigned)y * (unsigned)pitch + (unsigned)x
+                                 : (unsigned)wrap_near(y, ny) * (unsigned)pitch +
+                                       (((part >> i) & 1u) ? 0u : (unsigned)wrap_near(x, nx));
+            }
+            for (int k = aw; k < K; k += NA) {
+                const T* U = U0 + k * plane;
+                T* t = buf + k * PL + lane * VEC;
 #pragma unroll
                 for (int i = 0; i < NIT; ++i) {
-                    const int q = lane + 32 * i, r = q / CH, c = (q - r * CH) * VEC;
-                    const int y = y0 - 3 + r, x = x0 - 4 + c;
-                    so[i] = interior ? (unsigned)y * (unsigned)pitch + (unsigned)x
-                                     : (unsigned)wrap_near(y, ny) * (unsigned)pitch + (unsigned)wrap_near(x, nx);
+                    if ((whole >> i) & 1u) {
+                        const T* s = U + so[i];
+                        if (LBM_BC_NODE(cp, K, s - U0) && LBM_BC_NODE(cp, K, s - U0 + VEC - 1)) cp_async16(t + 32 * VEC * i, s);
+                    }
                 }
+            }
+            if (__any_sync(0xffffffffu, part != 0)) {
+#pragma unroll 1
                 for (int k = aw; k < K; k += NA) {
                     const T* U = U0 + k * plane;
                     T* t = buf + k * PL + lane * VEC;
 #pragma unroll
                     for (int i = 0; i < NIT; ++i) {
-                        if ((i + 1) * 32 <= RT * CH || lane + 32 * i < RT * CH) {
-                            const T* s = U + so[i];
-                            if (LBM_BC_NODE(cp, K, s - U0) && LBM_BC_NODE(cp, K, s - U0 + VEC - 1)) cp_async16(t + 32 * VEC * i, s);
+                        if ((part >> i) & 1u) {
+                            const int x = x0 - 4 + (lane + 32 * i) % CH * VEC;
+                            for (int e = 0; e < VEC; ++e) {
+                                const T* s = U + so[i] + (unsigned)wrap_near(x + e, nx);
+                                if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(t + 32 * VEC * i + e, s);
+                            }
                         }
-                    }
-                }
-            } else {
-                for (int k = aw; k < K; k += NA) {
-                    const T* U = U0 + k * plane;
-                    for (int i = lane; i < RT * HXP; i += 32) {
-                        const int r = i / HXP, c = i - r * HXP;
-                        const T* s = U + ((long long)wrap_near(y0 - 3 + r, ny) * pitch + wrap_near(x0 - 4 + c, nx));
-                        if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(buf + k * PL + i, s);
                     }
                 }
             }

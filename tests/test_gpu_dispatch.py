@@ -182,3 +182,19 @@ def test_fd_equilibrium_of_negative_density(q, scheme, prec):
     run = oracle.fd_imex_run if scheme == "imex" else oracle.fd_run
     ref = run(-f0, s.dx, s.dt, s.tau, 4)
     assert rel_err(got, ref) < (TOL64 if prec == "fp64" else 12 * 2 * 10 * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("prec,scheme", [("fp32", "rk3"), ("fp32", "imex"), ("fp64", "rk3")])
+@pytest.mark.parametrize("nx", [7, 29, 30, 31, 33, 34, 35, 61, 63, 65, 66, 99])
+def test_fd_ragged_width(nx, prec, scheme):
+    """Widths around a tile's edge with every remainder of a 16-byte copy: the
+    copies across the periodic edge and the ones left out beyond it. FP32
+    tolerance as above."""
+    f0 = _state(4, nx, 19, 17)
+    with _fd(4, nx, 19, scheme, prec) as L:
+        s = L.spec
+        L.set_populations(f0)
+        L.step(4)
+        got = L.populations()
+    run = oracle.fd_imex_run if scheme == "imex" else oracle.fd_run
+    assert rel_err(got, run(f0, s.dx, s.dt, s.tau, 4)) < (TOL64 if prec == "fp64" else 12 * 2 * 10 * 2.0 ** -24)
