@@ -432,27 +432,29 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             // 1. the K halo tiles of the stage input: 16-byte asynchronous
             //    copies (rows are 16-byte aligned: x0 - 4 is a multiple of 4, the
             //    pitch of 32). At the periodic edge a chunk wraps as a whole when
-            //    nx is a multiple of VEC; otherwise the chunks before x = 0 and
-            //    across nx go value by value, and those no node of the lattice
-            //    reaches (beyond nx + 2) are left out (whole edge tiles value by
-            //    value: FD 16-velocity 777 x 500 took 1.4x the time). A lane
-            //    copies the same chunks of every population's tile: their offsets
-            //    are formed once per item (below 2^32: a plane's elements times
-            //    the three buffers fit the device).
+            //    nx is a multiple of VEC; otherwise the few columns of the chunks
+            //    that cross it (before x = 0, and from the last chunk's start to
+            //    nx + 2) go value by value, spread over all preparing lanes, each
+            //    with one column's offset for all populations (wrapping every
+            //    value of every such chunk in the lane of its copy took half as
+            //    long again as the next width that is a multiple of 4: FD
+            //    16-velocity 750 x 322 FP32, 112 -> 74 us per step; 9-velocity
+            //    IMEX 68 -> 51). Columns that no node of the lattice reaches
+            //    (beyond nx + 2) are left out.
+            //    Offsets are below 2^32: a plane's elements times the three
+            //    buffers fit the device.
             const T* const U0 = static_cast<const T*>(cp->buf[in_idx]);
             const bool interior = x0 >= 4 && x0 + TX + 4 <= nx && y0 >= 3 && y0 + TY + 3 <= ny;
-            unsigned so[NIT], whole = 0, part = 0;   // one bit per chunk of the lane
+            unsigned so[NIT], whole = 0;   // one bit per chunk of the lane
 #pragma unroll
             for (int i = 0; i < NIT; ++i) {
                 const int q = lane + 32 * i, r = q / CH, c = (q - r * CH) * VEC;
                 const int y = y0 - 3 + r, x = x0 - 4 + c;
-                if ((i + 1) * 32 <= RT * CH || q < RT * CH) {
-                    if (interior || nx % VEC == 0 || (x >= 0 && x + VEC <= nx)) whole |= 1u << i;
-                    else if (x < nx + 3) part |= 1u << i;
-                }
+                if (((i + 1) * 32 <= RT * CH || q < RT * CH) &&
+                    (interior || (x < nx + 3 && (nx % VEC == 0 || (x >= 0 && x + VEC <= nx)))))
+                    whole |= 1u << i;
                 so[i] = interior ? (unsigned)y * (unsigned)pitch + (unsigned)x
-                                 : (unsigned)wrap_near(y, ny) * (unsigned)pitch +
-                                       (((part >> i) & 1u) ? 0u : (unsigned)wrap_near(x, nx));
+                                 : (unsigned)wrap_near(y, ny) * (unsigned)pitch + (unsigned)wrap_near(x, nx);
             }
             for (int k = aw; k < K; k += NA) {
                 const T* U = U0 + k * plane;
@@ -465,21 +467,17 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     }
                 }
             }
-            if (__any_sync(0xffffffffu, part != 0)) {
-#pragma unroll 1
-                for (int k = aw; k < K; k += NA) {
-                    const T* U = U0 + k * plane;
-                    T* t = buf + k * PL + lane * VEC;
-#pragma unroll
-                    for (int i = 0; i < NIT; ++i) {
-                        if ((part >> i) & 1u) {
-                            const int x = x0 - 4 + (lane + 32 * i) % CH * VEC;
-                            for (int e = 0; e < VEC; ++e) {
-                                const T* s = U + so[i] + (unsigned)wrap_near(x + e, nx);
-                                if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(t + 32 * VEC * i + e, s);
-                            }
-                        }
-                    }
+            if (nx % VEC != 0 && (x0 == 0 || x0 + TX + 3 > nx - nx % VEC)) {
+                const int xr = nx - nx % VEC;   // first column of the chunk across nx
+                const int nl = x0 == 0 ? 3 : 0, nr = max(min(nx + 3, x0 + TX + 3) - xr, 0);
+                for (int p = atid; p < RT * (nl + nr); p += NA * 32) {
+                    const int r = p / (nl + nr), e = p - r * (nl + nr);
+                    const int x = e < nl ? e - 3 : xr + e - nl;
+                    const T* s = U0 + ((unsigned)wrap_near(y0 - 3 + r, ny) * (unsigned)pitch + (unsigned)wrap_near(x, nx));
+                    T* t = buf + r * HXP + (x - x0 + 4);
+#pragma unroll 4
+                    for (int k = 0; k < K; ++k, s += plane, t += PL)
+                        if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(t, s);
                 }
             }
             // the next item's descriptor travels with the copies

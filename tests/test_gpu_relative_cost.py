@@ -1,0 +1,52 @@
+"""Calls that must not cost more than their neighbours: one run against a
+closely related one on the same GPU, in turn, as a ratio with a wide margin
+(absolute times depend on the machine)."""
+import time
+
+import pytest
+
+import lbm_workloads as wl
+import paper_1904_02471_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+VMAX = {3: 3 ** 0.5, 4: 2.33441421833897723932, 5: 2.85697001387280565416}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1904_02471_gb300 import build
+    build.build()
+    torch.cuda.init()
+
+
+def best_times(lattices, steps, rounds=7):
+    """Best time of `steps` steps of each lattice, the lattices in turn."""
+    best = [1e9] * len(lattices)
+    for r in range(rounds + 1):
+        for i, L in enumerate(lattices):
+            t = time.perf_counter()
+            L.step(steps)
+            L.sync()
+            if r:
+                best[i] = min(best[i], time.perf_counter() - t)
+    return best
+
+
+@pytest.mark.parametrize("q,nx,ny,scheme", [(4, 777, 500, "rk3"), (4, 750, 322, "rk3"), (3, 750, 322, "imex"), (3, 613, 249, "rk3")])
+def test_fd_ragged_width(q, nx, ny, scheme):
+    """FP32 FD rows whose length is no multiple of 4: the chunks across the
+    periodic edge are copied value by value. With the next multiple of 4 they
+    are not: the two cost the same to within a quarter."""
+    made = []
+    for n in (nx, (nx + 3) // 4 * 4):
+        dt = 0.3 / n / VMAX[q]
+        L = pkg.Lattice("fd", q, n, ny, dt / 5 if scheme == "imex" else 2 * dt, dt=dt, precision="fp32", scheme=scheme)
+        L.init(*wl.taylor_green(n, ny, 0.01))
+        made.append(L)
+    ragged, even = best_times(made, 64)
+    for L in made:
+        L.close()
+    assert ragged < 1.25 * even
