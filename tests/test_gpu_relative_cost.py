@@ -50,3 +50,22 @@ def test_fd_ragged_width(q, nx, ny, scheme):
     for L in made:
         L.close()
     assert ragged < 1.25 * even
+
+
+@pytest.mark.parametrize("nx,ny", [(88, 152), (131, 97)])
+def test_fd_default_tile_of_9_velocities(nx, ny):
+    """The tile picked by default against the configured ones, FD 9-velocity
+    lattices of one short tile per block: no configured tile is faster by a
+    twentieth."""
+    dt = 0.3 / nx / VMAX[3]
+    made = []
+    for tile in (None, 0, 1, 2, 3):
+        L = pkg.Lattice("fd", 3, nx, ny, 2 * dt, dt=dt, precision="fp32")
+        if tile is not None:
+            L.config(tile)
+        L.init(*wl.taylor_green(nx, ny, 0.01))
+        made.append(L)
+    t = best_times(made, 128)
+    for L in made:
+        L.close()
+    assert t[0] < 1.05 * min(t[1:])
