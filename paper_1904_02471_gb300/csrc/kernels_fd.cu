@@ -167,7 +167,9 @@ struct FdGeo {
     static constexpr int S = Q1 == 3 && sizeof(T) == 4 && H >= 2 ? 2 : 1;
     static constexpr int HS = H / S;
     static constexpr int NM = Q1 == 5 ? 13 : K * S;
-    static constexpr int NA = Q1 == 4 ? (IMEX ? 8 : 4) : (Q1 == 3 && S == 2 ? 4 : 7);
+    // IMEX prepares more: with four preparing warps 9 velocities take 575 us
+    // per step of 2048^2, with eight 494.
+    static constexpr int NA = Q1 == 4 || S == 2 ? (IMEX ? 8 : 4) : 7;
     static constexpr int NT = (NM + NA) * 32;
     // registers per thread of the two kinds of warps (FP32, 16 velocities: the
     // launch's registers are split between the warpgroups; 0: not split)
@@ -510,11 +512,23 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     Equil<T> e;
                     e.set(P::add(P::sp(r0), dr), dr, jx, jy);
                     const EquilAll<T, Q1> ea(e);
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        const V geq = P::mulc(ea.over_w(k), (T)w_of<Q1>(k));
-                        T* u = at(k, r, c);
-                        stv(u, P::mul(P::fma(vlam, geq, ldv_again(u)), vil));
+                    // map and sum the moments of Y (summed in a pass of their own,
+                    // they took 3 to 6% of a step); kept for the tile's own nodes
+                    set_moments<T, Q1>(
+                        [&](int k) {
+                            const V geq = P::mulc(ea.over_w(k), (T)w_of<Q1>(k));
+                            T* u = at(k, r, c);
+                            const V y = P::mul(P::fma(vlam, geq, ldv_again(u)), vil);
+                            stv(u, y);
+                            return y;
+                        },
+                        dr, jx, jy);
+                    if (r >= 0 && r < TY && c >= 0 && c < TX) {
+                        e.set(P::add(P::sp(r0), dr), dr, jx, jy);
+                        T* m = mo + 2 * (r * TX + c);
+                        stv2(m, e.px, e.py);
+                        stv2(m + 2 * TY * TX, e.jx, e.jy);
+                        stv(mo + 4 * TY * TX + r * TX + c, e.e0);
                     }
                 }
                 named_sync(1, NA * 32);
@@ -529,15 +543,18 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             for (int task = aw; task < H + NE; task += NA) {
                 if (task < H) {
                     const int r = task + grp * H;   // tile row
-                    V dr, jx, jy;
-                    set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c0)); }, dr, jx, jy);
-                    const V rho = P::add(P::sp(r0), dr);
-                    if (obs && y0 + r < ny) {
-                        const int pc = cp->probe_comp, y = y0 + r;
+                    T* m = mo + 2 * (r * TX + c0);
+                    Equil<T> e;
+                    if (!IMEX || obs) {
+                        V dr, jx, jy;
+                        set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c0)); }, dr, jx, jy);
+                        const V rho = P::add(P::sp(r0), dr);
+                        if (obs && y0 + r < ny) {
+                            const int pc = cp->probe_comp, y = y0 + r;
 #pragma unroll
-                        for (int h = 0; h < N; ++h) {
-                            const int x = x0 + c0 + h;
-                            if (x < nx) {
+                            for (int h = 0; h < N; ++h) {
+                                const int x = x0 + c0 + h;
+                                if (x >= nx) continue;
                                 acc[0] += P::get(dr, h);
                                 acc[1] += P::get(jx, h);
                                 acc[2] += P::get(jy, h);
@@ -554,9 +571,13 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                                 }
                             }
                         }
+                        if constexpr (!IMEX) e.set(rho, dr, jx, jy);
                     }
-                    Equil<T> e;
-                    e.set(rho, dr, jx, jy);
+                    if constexpr (IMEX) {
+                        ldv2(m, e.px, e.py);
+                        ldv2(m + 2 * TY * TX, e.jx, e.jy);
+                        e.e0 = ldv(mo + 4 * TY * TX + r * TX + c0);
+                    }
                     // FP32: residual moments of the collision term. In exact
                     // arithmetic sum_k (u_k - geq_k) (1, v_k) = 0; in float32 the
                     // rounding of the moments and of geq leaves a residual of
@@ -588,7 +609,6 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                         e.jx = P::add(e.jx, R1x);
                         e.jy = P::add(e.jy, R1y);
                     }
-                    T* m = mo + 2 * (r * TX + c0);
                     stv2(m, e.px, e.py);
                     stv2(m + 2 * TY * TX, e.jx, e.jy);
                     stv(mo + 4 * TY * TX + r * TX + c0, e.e0);
