@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     const int grp = lane / LC, c0 = (lane % LC) * N;   // row group and first column of the lane's nodes
     constexpr int DCH = sizeof(LatDesc) / 16;          // 16-byte chunks of a descriptor
     static_assert(sizeof(LatDesc) % 16 == 0 && DCH <= 32, "descriptors are copied in 16-byte chunks by one warp");
-    after_previous_launch();
+    wait_for_previous_launch();
     // a lone lattice's descriptor is read while the group's header is on its way
     if (tid < DCH) reinterpret_cast<uint4*>(s_desc)[tid] = reinterpret_cast<const uint4*>(g.desc)[tid];
     const int n_lat = g.hdr[0];
@@ -401,12 +401,13 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             }
             return item;
         };
-        // the item at or after `item` into slot s (one warp, asynchronous copy)
+        // the item at or after `item` into slot s (one warp, asynchronous copy;
+        // a lone lattice's descriptor is in slot 0 already)
         auto look_up = [&](int item, int s) {
             int li = 0;
             item = live_item(item, li);
             if (lane == 0) s_item[s] = item;
-            if (item < total && lane < DCH)
+            if (item < total && lane < DCH && (n_lat > 1 || s != 0))
                 cp_async16(reinterpret_cast<uint4*>(s_desc + s) + lane, reinterpret_cast<const uint4*>(g.desc + li) + lane);
         };
         constexpr int NIT = (RT * CH + 31) / 32;   // chunks of a population's tile per lane
@@ -423,6 +424,10 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             if (n >= NB) named_sync(4 + b, Ge::NT);
             const int item = s_item[slot];
             if (item >= total) {   // the march warps stop too
+                // a block takes its SM whole, so the next launch's blocks have
+                // no place before this one ends: let in at the start, they only
+                // kept SMs that were free from other streams (and 1 to 3% slower)
+                allow_next_launch();
                 named_arrive(2 + b, Ge::NT);
                 if (NB == 2 && n >= 1) named_sync(4 + (1 - b), Ge::NT);
                 break;

@@ -109,10 +109,13 @@ __device__ __forceinline__ void named_arrive(int id, int nthreads) {
 
 // Programmatic dependent launch. A step kernel's blocks may be on the SMs
 // before the launch they depend on has finished: every thread waits for it (and
-// for its writes) first, then lets the next launch come.
+// for its writes) first, then lets the next launch come (once every block has,
+// or has ended).
+__device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_previous_launch() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_previous_launch();
+    allow_next_launch();
 }
 
 // Change the registers per thread of the calling warpgroup (four aligned
