@@ -162,13 +162,23 @@ int Engine::default_grid(const Group& g, int tile) const {
     return persistent_grid(g, tile) * std::max(1, grid_mult_);
 }
 
+// Cost of an FD tile beside its rows (halo, moments, first faces, block start),
+// in rows, per kind of kernel: from the times of every tile on 29 lattices (FP64:
+// 9) from 20 x 20 to 2048^2, 9, 16 and 25 velocities. The pick of default_tile is
+// the fastest tile or within 4% of it (FP32 RK3: 7%) on each of them; one
+// constant for all, from 16-velocity RK3 tiles alone, missed by up to 19%
+// (blocked step, 333 x 217: 8 rows where 16 are faster).
+static double tile_row_cost(const Group& g) {
+    const bool fp64 = g.precision == LBM_FP64;
+    if (g.scheme == LBM_TS_RK3_FUSED) return fp64 ? 6 : 18;   // 18 halo rows
+    if (g.scheme == LBM_TS_IMEX) return fp64 ? 1.4 : 6.4;
+    return fp64 ? 0.8 : (g.q1 == 4 ? 3.5 : 6.4);
+}
+
 // Default tile of a group. FD: the variant with the least rounds x (rows + c),
-// rounds = tiles per SM rounded up, c the cost of a tile beside its rows (halo,
-// moments, first faces, block start) in rows. Measured per tile and stage, 16
-// velocities: FP32 4.96 / 2.92 / 2.17 / 1.95 us and FP64 204 / 110 / 64 / 40 us
-// with 16 / 8 / 4 / 2 rows: c = 6.4 and 1.4. Small lattices get small tiles
-// (more SMs at work: FP64 60^2, 35 us per step with 1 row, 48 with 2), large
-// ones tall tiles (FP32 2048^2, 0.80 ms per step with 16 rows, 0.95 with 8).
+// rounds = tiles per SM rounded up, c = tile_row_cost. Small lattices get small
+// tiles (more SMs at work: FP64 60^2, 35 us per step with 1 row, 48 with 2),
+// large ones tall tiles (FP32 2048^2, 0.78 ms per step with 16 rows, 0.90 with 8).
 // CS: the bulk-copy kernel where the state streams through HBM (FP32, in place:
 // 198 us per step of 4096^2 against 225 for the plain kernel), else the plain
 // one: a bulk tile of 32 rows is a chain of 32 row copies on one SM (256^2: 24
@@ -187,7 +197,7 @@ int Engine::default_tile(const Group& g) const {
         if (g.precision == LBM_FP32_DEV) return nodes >= 8LL << 20 ? (int)CS_B256x32 : (int)CS_T128x1;
         return nodes <= 128LL * sm_count_ ? (int)CS_T32x1 : (nodes < 65536 ? (int)CS_T128x1 : (int)CS_T128x2);
     }
-    const double c = g.precision == LBM_FP64 ? 1.4 : 6.4;
+    const double c = tile_row_cost(g);
     int best = g.tile;
     double best_cost = 1e300;
     for (int t = 0; t < (int)FD_NALL; ++t) {

@@ -52,20 +52,25 @@ def test_fd_ragged_width(q, nx, ny, scheme):
     assert ragged < 1.25 * even
 
 
-@pytest.mark.parametrize("nx,ny", [(88, 152), (131, 97)])
-def test_fd_default_tile_of_9_velocities(nx, ny):
-    """The tile picked by default against the configured ones, FD 9-velocity
-    lattices of one short tile per block: no configured tile is faster by a
-    twentieth."""
-    dt = 0.3 / nx / VMAX[3]
+@pytest.mark.parametrize("q,nx,ny,prec,scheme", [(3, 88, 152, "fp32", "rk3"), (3, 131, 97, "fp32", "rk3"),
+                                                 (4, 333, 217, "fp32", "rk3_fused"), (5, 257, 129, "fp32", "rk3_fused"),
+                                                 (5, 400, 400, "fp64", "rk3")])
+def test_fd_default_tile(q, nx, ny, prec, scheme):
+    """The tile picked by default against the configured ones: none of them is
+    faster by a twentieth."""
+    dt = 0.3 / nx / VMAX[q]
     made = []
     for tile in (None, 0, 1, 2, 3):
-        L = pkg.Lattice("fd", 3, nx, ny, 2 * dt, dt=dt, precision="fp32")
+        L = pkg.Lattice("fd", q, nx, ny, 2 * dt, dt=dt, precision=prec, scheme=scheme)
         if tile is not None:
-            L.config(tile)
+            try:
+                L.config(tile)
+            except pkg.LbmError:   # a tile that does not fit this set and precision
+                L.close()
+                continue
         L.init(*wl.taylor_green(nx, ny, 0.01))
         made.append(L)
-    t = best_times(made, 128)
+    t = best_times(made, 128 if prec == "fp32" else 8)
     for L in made:
         L.close()
     assert t[0] < 1.05 * min(t[1:])
