@@ -525,7 +525,7 @@ int Engine::enqueue_chunk(int c) {
             auto finish = [&]() -> cudaError_t {
                 if (!obs_launch(g)) return cudaSuccess;
                 ++n;
-                return launch_obs_finish(gd, (int)g.members.size(), g.obs_rows(), g.grid, j, stream_);
+                return launch_obs_finish(gd, (int)g.members.size(), g.total_items, g.grid, j, stream_);
             };
             if (g.model == LBM_CS) {
                 e = launch_cs_step(g.precision, g.tile, g.grid, gd, j, stream_);
@@ -646,7 +646,7 @@ int Engine::step_profiled(long long n, double* ms, int cap, double* total_ms) {
                     cudaEvent_t c = ev(), d = ev();
                     if (!c || !d) { cleanup(); return cuda_fail(cudaGetLastError(), "cudaEventCreate"); }
                     cudaEventRecord(c, stream_);
-                    e = launch_obs_finish(gd, (int)g.members.size(), g.obs_rows(), g.grid, 0, stream_);
+                    e = launch_obs_finish(gd, (int)g.members.size(), g.total_items, g.grid, 0, stream_);
                     cudaEventRecord(d, stream_);
                     if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "profiled finalize"); }
                     ++launches_;

@@ -77,7 +77,7 @@ bool fd_variant_fits(int precision, int q1, int tile, int scheme);
 
 // Observables of the lattices observed at sub-step j, after a step kernel
 // launched with `grid` blocks that did not finish them (finish_obs = 0).
-cudaError_t launch_obs_finish(const GroupDev& g, int lattices, int rows, int grid, int j, cudaStream_t s);
+cudaError_t launch_obs_finish(const GroupDev& g, int lattices, int items, int grid, int j, cudaStream_t s);
 // Advance steps/phase of every lattice by min(remaining, c).
 cudaError_t launch_advance(const GroupDev& g, int max_lat, int c, int flip_phase, cudaStream_t s);
 

@@ -74,3 +74,25 @@ def test_fd_default_tile(q, nx, ny, prec, scheme):
     for L in made:
         L.close()
     assert t[0] < 1.05 * min(t[1:])
+
+
+@pytest.mark.parametrize("model", ["cs", "fd"])
+def test_recording_many_lattices(model):
+    """A set of small lattices with the observables of every step recorded:
+    beside the step itself that is four sums per tile and their finishing,
+    not more than twice the step again."""
+    side, count = 32, 2000
+    dt = 0.3 / side / VMAX[3]
+    spec = pkg.make_spec(model, 3, side, side, 0.5 if model == "cs" else 2 * dt, 0.0 if model == "cs" else dt, 0.0, "fp32")
+    made = []
+    for every in (1, 0):
+        B = pkg.Batch([spec] * count)
+        for i in range(count):
+            B.init(i, *wl.taylor_green(side, side, 0.01))
+            if every:
+                B.record(i, every, 1 << 10)
+        made.append(B)
+    recorded, plain = best_times(made, 16, rounds=4)
+    for B in made:
+        B.close()
+    assert recorded < 3 * plain
