@@ -179,23 +179,39 @@ static double tile_row_cost(const Group& g) {
 // rounds = tiles per SM rounded up, c = tile_row_cost. Small lattices get small
 // tiles (more SMs at work: FP64 60^2, 35 us per step with 1 row, 48 with 2),
 // large ones tall tiles (FP32 2048^2, 0.78 ms per step with 16 rows, 0.90 with 8).
-// CS: the bulk-copy kernel where the state streams through HBM (FP32, in place:
-// 198 us per step of 4096^2 against 225 for the plain kernel), else the plain
-// one: a bulk tile of 32 rows is a chain of 32 row copies on one SM (256^2: 24
-// us per step, plain 2.8; 1024^2: 25 and 13; 2048^2: 60.6 and 58.9). FP64 is
+// CS FP32: the bulk-copy kernel where the state streams through HBM (in place: 198
+// us per step of 4096^2 against 225 for the plain kernel; the lines lie at 2400^2:
+// 2300^2 in place 71 and 73, 2500^2 86 and 88), else the plain one: a bulk tile of
+// 32 rows is a chain of 32 row copies on one SM (256^2: 24 us per step, plain 2.8;
+// 1024^2: 25 and 13; 2048^2: 60.6 and 58.9). A plain block of one row leaves a row
+// of sums for every 128 nodes, a bulk tile one for 8192: with observables every
+// few steps the bulk kernel is ahead from 1.6 Mi nodes on (1448^2, every step: 43
+// us per step, plain 61; every 8th: 35 and 40; 2880^2 every step 121 and 193), and
+// the plain tile of 4 rows below (1000 x 777, every step: 24 and 28). Sets of
+// lattices and narrow ones get tiles 64 wide (200 of 64^2: 18 us per step, 27 with
+// 128 x 1; 31 x 20000: 18 and 24), in large sets and lattices of them the
+// narrower bulk tile (2000 of 64^2: 198, 310 with 128 x 1, 212 with 256 x 32). FP64 is
 // bound by the FP64 pipe, so its tiles spread over the SMs: one row of 32
 // nodes while all of them fit the GPU at once, then 128 x 1, then 128 x 2
 // (256^2: 11.1 us per step against 11.3 and 141 with bulk tiles).
 int Engine::default_tile(const Group& g) const {
     if (g.model == LBM_CS) {
         long long nodes = 0;
-        for (int li : g.members) nodes += (long long)lat[li].spec.nx * lat[li].spec.ny;
+        int widest = 0;
+        for (int li : g.members) {
+            nodes += (long long)lat[li].spec.nx * lat[li].spec.ny;
+            widest = std::max(widest, lat[li].spec.nx);
+        }
         // the injection needs the kernel that waits; a server keeps it too: its
         // test of overlapping runs counts on a run of 4000 CS steps on 512^2
         // still being on the GPU after 50 ms (plain tiles end it after 30)
         if (inject_us_ > 0 || dynamic_) return (int)CS_B256x32;
-        if (g.precision == LBM_FP32_DEV) return nodes >= 8LL << 20 ? (int)CS_B256x32 : (int)CS_T128x1;
-        return nodes <= 128LL * sm_count_ ? (int)CS_T32x1 : (nodes < 65536 ? (int)CS_T128x1 : (int)CS_T128x2);
+        if (g.precision == LBM_FP64)
+            return nodes <= 128LL * sm_count_ ? (int)CS_T32x1 : (nodes < 65536 ? (int)CS_T128x1 : (int)CS_T128x2);
+        const bool often = g.min_every > 0 && g.min_every <= 16;
+        if (nodes >= (often ? 3LL << 19 : 11LL << 19)) return widest <= 64 ? (int)CS_B128x32 : (int)CS_B256x32;
+        const bool narrow = g.members.size() > 1 || widest <= 64;
+        return nodes >= 1 << 17 && (narrow || often) ? (int)CS_T64x4 : (int)CS_T128x1;
     }
     const double c = tile_row_cost(g);
     int best = g.tile;
@@ -400,8 +416,13 @@ LatDesc Engine::make_desc(const Lattice& L, const Group& g, int item_begin, doub
 
 int Engine::upload_group(int gi) {
     Group& g = groups[gi];
-    if (dynamic_ && g.auto_tile && !g.members.empty()) {
-        // the lattices come and go: the tile follows them
+    g.min_every = 0;
+    for (int li : g.members)
+        if (lat[li].obs_every > 0)
+            g.min_every = g.min_every > 0 ? std::min(g.min_every, lat[li].obs_every) : lat[li].obs_every;
+    if ((dynamic_ || g.model == LBM_CS) && g.auto_tile && !g.members.empty()) {
+        // the tile follows the lattices of a server as they come and go, and CS
+        // recording
         const int tile = default_tile(g);
         if (tile != g.tile) {
             g.tile = tile;
@@ -413,10 +434,8 @@ int Engine::upload_group(int gi) {
     const int ty = g.model == LBM_CS ? cs_tile_ty(g.tile) : fd_tile_ty(g.tile);
     std::vector<int> begins;
     long long items = 0;
-    g.min_every = 0;
     for (int li : g.members) {
         const Lattice& L = lat[li];
-        if (L.obs_every > 0) g.min_every = g.min_every > 0 ? std::min(g.min_every, L.obs_every) : L.obs_every;
         begins.push_back((int)items);
         items += (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty);
     }

@@ -96,3 +96,38 @@ def test_recording_many_lattices(model):
     for B in made:
         B.close()
     assert recorded < 3 * plain
+
+
+@pytest.mark.parametrize("storage", ["ab", "inplace"])
+def test_recording_a_cs_lattice_every_step(storage):
+    """The observables of every step cost a CS lattice of ordinary size less
+    than a third of a step."""
+    made = []
+    for every in (1, 0):
+        L = pkg.Lattice("cs", 3, 2500, 2500, 0.5, precision="fp32", storage=storage)
+        L.init(*wl.taylor_green(2500, 2500, 0.01))
+        if every:
+            L.record(every, 1 << 10)
+        made.append(L)
+    recorded, plain = best_times(made, 32)
+    for L in made:
+        L.close()
+    assert recorded < 4 / 3 * plain
+
+
+@pytest.mark.parametrize("side,count,every", [(32, 200, 1), (32, 2000, 0), (64, 2000, 0), (64, 2000, 1), (256, 120, 0)])
+def test_cs_default_tile_of_a_set(side, count, every):
+    """The tile picked by default for a set of CS lattices against the
+    configured ones: none of them is faster by a fifth."""
+    spec = pkg.make_spec("cs", 3, side, side, 0.5, 0.0, 0.0, "fp32")
+    B = pkg.Batch([spec] * count)
+    for i in range(count):
+        B.init(i, *wl.taylor_green(side, side, 0.01))
+        if every:
+            B.record(i, every, 1 << 12)
+    t = best_times([B], 16, rounds=4)
+    for tile in (0, 2, 4, 5, 6):
+        B.config(0, tile)
+        t += best_times([B], 16, rounds=4)
+    B.close()
+    assert t[0] < 1.2 * min(t[1:])
