@@ -202,12 +202,16 @@ int Engine::default_tile(const Group& g) const {
             nodes += (long long)lat[li].spec.nx * lat[li].spec.ny;
             widest = std::max(widest, lat[li].spec.nx);
         }
-        // the injection needs the kernel that waits; a server keeps it too: its
-        // test of overlapping runs counts on a run of 4000 CS steps on 512^2
-        // still being on the GPU after 50 ms (plain tiles end it after 30)
-        if (inject_us_ > 0 || dynamic_) return (int)CS_B256x32;
+        // The injection needs the kernel that waits. A server's larger sets keep it
+        // too, only because its test of overlapping runs counts on a run of 4000 CS
+        // steps on 512^2 still being on the GPU after 50 ms (plain tiles end it
+        // after 30); its smaller ones take plain tiles (20000 steps of 64^2: 24 us
+        // each with bulk tiles), the same for FP32 whatever comes and goes, so
+        // that the captured graph stays.
+        if (inject_us_ > 0 || (dynamic_ && nodes >= 1 << 18)) return (int)CS_B256x32;
         if (g.precision == LBM_FP64)
             return nodes <= 128LL * sm_count_ ? (int)CS_T32x1 : (nodes < 65536 ? (int)CS_T128x1 : (int)CS_T128x2);
+        if (dynamic_) return (int)CS_T128x1;
         const bool often = g.min_every > 0 && g.min_every <= 16;
         if (nodes >= (often ? 3LL << 19 : 11LL << 19)) return widest <= 64 ? (int)CS_B128x32 : (int)CS_B256x32;
         const bool narrow = g.members.size() > 1 || widest <= 64;

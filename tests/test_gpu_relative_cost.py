@@ -7,6 +7,7 @@ import pytest
 
 import lbm_workloads as wl
 import paper_1904_02471_gb300 as pkg
+from paper_1904_02471_gb300 import lbm
 
 pytestmark = pytest.mark.gpu
 
@@ -131,3 +132,22 @@ def test_cs_default_tile_of_a_set(side, count, every):
         t += best_times([B], 16, rounds=4)
     B.close()
     assert t[0] < 1.2 * min(t[1:])
+
+
+def test_served_run_of_a_small_cs_lattice():
+    """A CS run of many steps on a small lattice, served alone, against the same
+    steps of a lattice of its own: rounds of 256 steps and their bookkeeping
+    cost less than three times the steps again."""
+    n, steps = 64, 20000
+    spec = pkg.make_spec("cs", 3, n, n, 0.5, 0.0, 0.0, "fp32")
+    with lbm.Server(1 << 30, 4, 256) as S:
+        S.submit(lbm.make_request(spec, 256, "tg", 0.01))
+        S.drain(60)
+        t = time.perf_counter()
+        S.submit(lbm.make_request(spec, steps, "tg", 0.01))
+        S.drain(60)
+        served = time.perf_counter() - t
+    with pkg.Lattice("cs", 3, n, n, 0.5, precision="fp32") as L:
+        L.init(*wl.taylor_green(n, n, 0.01))
+        alone = best_times([L], steps, rounds=2)[0]
+    assert served < 4 * alone
