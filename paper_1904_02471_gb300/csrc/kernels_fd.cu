@@ -81,7 +81,7 @@ struct Equil {
     __device__ __forceinline__ void set(V rho, V dr, V jx_, V jy_) {
         jx = jx_;
         jy = jy_;
-        const V h = P::mulc(P::rcp(rho), T(0.5));
+        const V h = P::mulc(P::rcp_node(rho), T(0.5));
         px = P::mul(jx, h);
         py = P::mul(jy, h);
         e0 = P::fma(P::neg(jy), py, P::fma(P::neg(jx), px, dr));
