@@ -330,25 +330,17 @@ __device__ __forceinline__ void obs_add_group(const LatDesc& d, int g, int rows,
             make_obs(step, d.dt, d.nx, d.ny, d.rho0, d.probe_comp, d.probe_norm, tot);
     }
 }
-// A block's tile `local` of an observed lattice: the threads' sums v are added
-// up (warp level in T: at most 32 per-thread sums in float; across warps and
-// tiles in double, in threads below NOBS) and the block's last tile of the
-// lattice stores its row. With `finish` the block that completes OBS_GROUP
+// A block's tile `local` of an observed lattice, its warps' sums in red[warp]
+// [NOBS]: they are added up (across warps and tiles in double, in threads below
+// NOBS) and the block's last tile of the lattice stores its row. With `finish` the block that completes OBS_GROUP
 // rows goes on as above: no launch after the step (two such launches took 5 us
 // of every recorded step of a small lattice). Without it a launch of
 // obs_finish_kernel does: where a launch has thousands of blocks, a fence and
 // a count in each of them cost more (CS 8192^2: 0.767 ms per step against
 // 0.745).
-template <typename T, int NT, typename Sync>
-__device__ __forceinline__ void obs_tile(const T (&v)[NOBS], const LatDesc& d, int local, long long step, int tid,
-                                         double& run, double* red, int* flag, Sync sync, bool finish) {
-#pragma unroll
-    for (int q = 0; q < NOBS; ++q) {
-        T x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if ((tid & 31) == 0) red[(tid >> 5) * NOBS + q] = (double)x;
-    }
+template <int NT, typename Sync>
+__device__ __forceinline__ void obs_warp_sums(const LatDesc& d, int local, long long step, int tid, double& run,
+                                              double* red, int* flag, Sync sync, bool finish) {
     sync();
     const int grid = (int)gridDim.x;
     if (tid < NOBS) {
@@ -365,6 +357,21 @@ __device__ __forceinline__ void obs_tile(const T (&v)[NOBS], const LatDesc& d, i
         }
     }
     sync();   // red and flag are free again
+}
+// The same from the threads' sums v, added up per warp in T: 32 of them in
+// float, each of them a float sum over the thread's nodes (CS: 1 to 4, bulk
+// tiles up to 32; temporally blocked FD step: 1).
+template <typename T, int NT, typename Sync>
+__device__ __forceinline__ void obs_tile(const T (&v)[NOBS], const LatDesc& d, int local, long long step, int tid,
+                                         double& run, double* red, int* flag, Sync sync, bool finish) {
+#pragma unroll
+    for (int q = 0; q < NOBS; ++q) {
+        T x = v[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((tid & 31) == 0) red[(tid >> 5) * NOBS + q] = (double)x;
+    }
+    obs_warp_sums<NT>(d, local, step, tid, run, red, flag, sync, finish);
 }
 
 }  // namespace lbm

@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             // 2. per warp, one of: the moments of a row of each group (Eq.
             //    f_moments_discrete) with the observables of the state; the
             //    faces beyond the outermost lane, one (population, rows) per lane
-            T acc[NOBS] = {T(0), T(0), T(0), T(0)};
+            double sum = 0.0;   // of observable `lane` over the warp's nodes
             constexpr int KX = Q1 * (Q1 - Q1 % 2);   // populations with faces along x
             constexpr int NE = (KX * H + 31) / 32;
             for (int task = aw; task < H + NE; task += NA) {
@@ -554,26 +554,37 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                         V dr, jx, jy;
                         set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c0)); }, dr, jx, jy);
                         const V rho = P::add(P::sp(r0), dr);
-                        if (obs && y0 + r < ny) {
+                        if (obs) {
+                            // one node of each lane is added up per warp in T (32
+                            // float values, as with a node per thread), the rest
+                            // in double
                             const int pc = cp->probe_comp, y = y0 + r;
 #pragma unroll
                             for (int h = 0; h < N; ++h) {
                                 const int x = x0 + c0 + h;
-                                if (x >= nx) continue;
-                                acc[0] += P::get(dr, h);
-                                acc[1] += P::get(jx, h);
-                                acc[2] += P::get(jy, h);
-                                if (pc >= 0) {
-                                    T pxv, pyv;
-                                    if constexpr (sizeof(T) == 4) {
-                                        pxv = cp->probe_pxf[x];
-                                        pyv = cp->probe_pyf[y];
-                                    } else {
-                                        pxv = cp->probe_px[x];
-                                        pyv = cp->probe_py[y];
+                                T v[NOBS] = {T(0), T(0), T(0), T(0)};
+                                if (x < nx && y < ny) {
+                                    v[0] = P::get(dr, h);
+                                    v[1] = P::get(jx, h);
+                                    v[2] = P::get(jy, h);
+                                    if (pc >= 0) {
+                                        T pxv, pyv;
+                                        if constexpr (sizeof(T) == 4) {
+                                            pxv = cp->probe_pxf[x];
+                                            pyv = cp->probe_pyf[y];
+                                        } else {
+                                            pxv = cp->probe_px[x];
+                                            pyv = cp->probe_py[y];
+                                        }
+                                        v[3] = (pc == 0 ? P::get(jx, h) : P::get(jy, h)) / P::get(rho, h) * pxv * pyv;
                                     }
-                                    acc[3] += (pc == 0 ? P::get(jx, h) : P::get(jy, h)) / P::get(rho, h) * pxv * pyv;
                                 }
+#pragma unroll
+                                for (int q = 0; q < NOBS; ++q) {
+#pragma unroll
+                                    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+                                }
+                                sum += (double)(lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3]);
                             }
                         }
                         if constexpr (!IMEX) e.set(rho, dr, jx, jy);
@@ -635,9 +646,11 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     }
                 }
             }
-            if (obs)
-                obs_tile<T, NA * 32>(acc, *cp, local, cp->step0 + j, atid, run, red, &s_last,
-                                     [] { named_sync(1, NA * 32); }, g.finish_obs != 0);
+            if (obs) {
+                if (lane < NOBS) red[aw * NOBS + lane] = sum;
+                obs_warp_sums<NA * 32>(*cp, local, cp->step0 + j, atid, run, red, &s_last,
+                                       [] { named_sync(1, NA * 32); }, g.finish_obs != 0);
+            }
             named_arrive(2 + b, Ge::NT);
         }
         return;
