@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             // (`total` or beyond: none), and that lattice
             for (; item < total; item += gridDim.x) {
                 li = 0;
-                int first = 0, end = total;
+                int end = total;
                 bool dead;
                 if (n_lat == 1) {
                     dead = (long long)j >= s_desc[0].remaining;
@@ -387,14 +387,12 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                         if (s_begin[mid] <= item) li = mid;
                         else hi = mid - 1;
                     }
-                    first = s_begin[li];
                     if (li + 1 < n_lat) end = s_begin[li + 1];
                     dead = s_dead[li];
                 } else {
-                    li = find_lattice(g.item_begin, n_lat, item);
-                    first = g.desc[li].item_begin;
-                    end = first + g.desc[li].items;
+                    li = find_lattice_warp(g.item_begin, n_lat, item, lane);
                     dead = (long long)j >= g.desc[li].remaining;
+                    if (dead) end = g.desc[li].item_begin + g.desc[li].items;
                 }
                 if (!dead) break;
                 item += (end - 1 - item) / (int)gridDim.x * (int)gridDim.x;   // passed over in one jump

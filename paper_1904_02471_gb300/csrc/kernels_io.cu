@@ -171,14 +171,10 @@ __global__ void __launch_bounds__(FIN_THREADS) obs_finish_kernel(GroupDev g, int
     __shared__ double red[FIN_THREADS / 32 * NOBS];
     __shared__ int s_last;
     after_previous_launch();
+    const int n_lat = g.hdr[0];
     auto first_block = [&](int i) { return g.item_begin[i] / OBS_GROUP + i; };
-    int li = 0;
-    for (int hi = g.hdr[0] - 1; li < hi;) {
-        const int mid = (li + hi + 1) >> 1;
-        if (first_block(mid) <= (int)blockIdx.x) li = mid;
-        else hi = mid - 1;
-    }
-    if (li >= g.hdr[0]) return;
+    const int li = last_at_most(n_lat, threadIdx.x & 31, [&](int i) { return first_block(i) <= (int)blockIdx.x; });
+    if (li >= n_lat) return;
     const LatDesc& d = g.desc[li];
     const int gr = (int)blockIdx.x - first_block(li);
     if ((long long)j >= d.remaining || !observe_now(d, j)) return;

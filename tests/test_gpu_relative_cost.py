@@ -151,3 +151,24 @@ def test_served_run_of_a_small_cs_lattice():
         L.init(*wl.taylor_green(n, n, 0.01))
         alone = best_times([L], steps, rounds=2)[0]
     assert served < 4 * alone
+
+
+def _fd_set(count, side, every=0):
+    dt = 0.3 / side / VMAX[3]
+    B = pkg.Batch([pkg.make_spec("fd", 3, side, side, 2 * dt, dt, 0.0, "fp32")] * count)
+    for i in range(count):
+        B.init(i, *wl.taylor_green(side, side, 0.01))
+        if every:
+            B.record(i, every, 1 << 12)
+    return B
+
+
+def test_fd_set_beyond_the_lookup_table():
+    """Up to 256 lattices of a set are looked up in shared memory, more in global
+    memory. 256 and 300 lattices of two tiles are four rounds of tiles each: the
+    same time to within a twelfth."""
+    made = [_fd_set(256, 32), _fd_set(300, 32)]
+    table, beyond = best_times(made, 64, rounds=9)
+    for B in made:
+        B.close()
+    assert beyond < 13 / 12 * table
