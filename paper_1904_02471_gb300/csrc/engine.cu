@@ -438,10 +438,13 @@ int Engine::upload_group(int gi) {
     const int ty = g.model == LBM_CS ? cs_tile_ty(g.tile) : fd_tile_ty(g.tile);
     std::vector<int> begins;
     long long items = 0;
+    g.items.clear();
     for (int li : g.members) {
         const Lattice& L = lat[li];
         begins.push_back((int)items);
-        items += (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty);
+        const long long own = (long long)((L.spec.nx + tx - 1) / tx) * ((L.spec.ny + ty - 1) / ty);
+        g.items.push_back((int)std::min(own, 1LL << 30));
+        items += own;
     }
     if (items >= (1LL << 31)) { set_error("too many work items"); return LBM_EINVAL; }
     const int nm = (int)g.members.size();

@@ -87,6 +87,7 @@ struct Group {
     bool auto_tile = true;   // the tile is the default one (no configuration, no tuning)
     int grid = 0;
     std::vector<int> members;
+    std::vector<int> items;   // of the members
     // two allocations, at d_desc (descriptors, header words, first items) and
     // at d_partials (tile partials, group sums, counters)
     LatDesc* d_desc = nullptr;
@@ -99,16 +100,28 @@ struct Group {
     double* d_group_partials = nullptr;   // [sum of obs_groups][NOBS]
     unsigned* d_obs_count = nullptr;      // [sum of obs_groups + 1]
     bool overlap = true;        // launches may overlap (launch_overlapped)
-    // rows of partial sums of a launch (at most)
-    int obs_rows() const { return grid < total_items ? grid : total_items; }
+    // rows of partial sums of a launch, over all lattices (each has one per
+    // block that does any of its tiles)
+    long long obs_rows() const {
+        long long rows = 0;
+        for (int n : items) rows += n < grid ? n : grid;
+        return rows;
+    }
     // shortest recording interval of the members (0: none records)
     long long min_every = 0;
     // the step kernels finish the observables themselves, unless thousands of
     // rows are recorded every few steps: a launch after every step then costs
     // less than counting them (CS 8192^2, every step: 7 us against 22; CS
-    // 1000 x 777, every 20th: 0.8 us per step against nothing). A server's
-    // always do: its items change under a captured graph.
-    bool finish_obs() const { return !overlap || obs_rows() <= 4096 || min_every >= 4; }
+    // 1000 x 777, every 20th: 0.8 us per step against nothing), and likewise
+    // where a block has rows of several lattices, each with its count (FD: 48
+    // lattices of 128^2, 9 velocities, every step: 177 us per step against 149).
+    // A server's always do: its items change under a captured graph.
+    bool finish_obs() const {
+        if (!overlap) return true;
+        const long long rows = obs_rows(), blocks = grid < total_items ? grid : total_items;
+        if (2 * rows > blocks * (min_every > 2 ? min_every : 2)) return false;
+        return rows <= 4096 || min_every >= 4;
+    }
     GroupDev dev() const { return GroupDev{d_desc, d_item_begin, d_hdr, finish_obs() ? 1 : 0, overlap ? 1 : 0}; }
 };
 

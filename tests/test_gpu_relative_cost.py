@@ -172,3 +172,12 @@ def test_fd_set_beyond_the_lookup_table():
     for B in made:
         B.close()
     assert beyond < 13 / 12 * table
+
+
+def test_recording_an_fd_set_every_step():
+    """Observables of every step: one of the three stages sums them up."""
+    made = [_fd_set(48, 128, 1), _fd_set(48, 128)]
+    recorded, plain = best_times(made, 32)
+    for B in made:
+        B.close()
+    assert recorded < 4 / 3 * plain
