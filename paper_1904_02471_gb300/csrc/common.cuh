@@ -233,36 +233,36 @@ __device__ __forceinline__ double fast_rcp(double x) {
     return ::fma(::fma(e, e, e), r, r);
 }
 
-// Block reduction of NOBS per-thread partial sums into out[NOBS] (double).
-// Warp level in T (for FP32 storage: at most 32 per-thread sums in float),
-// across warps in double, fixed order (deterministic).
-// Must be called by all threads of the block. With TRAILING_SYNC false the
-// caller guarantees a barrier before `smem` is written again.
-template <typename T, int NT, bool TRAILING_SYNC = true>
-__device__ __forceinline__ void block_reduce_obs(const T (&v)[NOBS], double* out, double* smem) {
-    constexpr int NW = NT / 32;
-    T r[NOBS];
+// The sums of NOBS values per lane over a warp, one of them in each lane (number
+// obs_of_lane): 6 shuffles and additions, each quantity added up in a tree of 32
+// values (with a butterfly for each of the four there are 20).
+__device__ __forceinline__ int obs_of_lane(int lane) { return (lane & 1) * 2 + (lane >> 1 & 1); }
+template <typename T>
+__device__ __forceinline__ T warp_obs_sums(const T (&v)[NOBS], int lane) {
+    static_assert(NOBS == 4, "two halvings");
+    const bool b0 = lane & 1, b1 = lane & 2;
+    const T a0 = (b0 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, b0 ? v[0] : v[2], 1);
+    const T a1 = (b0 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, b0 ? v[1] : v[3], 1);
+    T a = (b1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b1 ? a0 : a1, 2);
 #pragma unroll
-    for (int q = 0; q < NOBS; ++q) {
-        T x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        r[q] = x;
-    }
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < NOBS; ++q) smem[warp * NOBS + q] = (double)r[q];
+    for (int o = 4; o <= 16; o *= 2) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+// Block reduction of NOBS per-thread partial sums into out[NOBS], in a fixed
+// order. Must be called by all threads of the block.
+template <int NT>
+__device__ __forceinline__ void block_reduce_obs(const double (&v)[NOBS], double* out, double* smem) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double x = warp_obs_sums(v, lane);
+    if (lane < NOBS) smem[warp * NOBS + obs_of_lane(lane)] = x;
+    __syncthreads();
+    if (threadIdx.x < NOBS) {
+        double s = 0.0;
+        for (int w = 0; w < NT / 32; ++w) s += smem[w * NOBS + threadIdx.x];
+        out[threadIdx.x] = s;
     }
     __syncthreads();
-    if (tid < NOBS) {
-        double s = 0.0;
-        for (int w = 0; w < NW; ++w) s += smem[w * NOBS + tid];
-        out[tid] = s;
-    }
-    if constexpr (TRAILING_SYNC) __syncthreads();
 }
 
 // The observables record of a state from its NOBS global sums.
@@ -384,13 +384,9 @@ __device__ __forceinline__ void obs_warp_sums(const LatDesc& d, int local, long 
 template <typename T, int NT, typename Sync>
 __device__ __forceinline__ void obs_tile(const T (&v)[NOBS], const LatDesc& d, int local, long long step, int tid,
                                          double& run, double* red, int* flag, Sync sync, bool finish) {
-#pragma unroll
-    for (int q = 0; q < NOBS; ++q) {
-        T x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if ((tid & 31) == 0) red[(tid >> 5) * NOBS + q] = (double)x;
-    }
+    const int lane = tid & 31;
+    const T x = warp_obs_sums(v, lane);
+    if (lane < NOBS) red[(tid >> 5) * NOBS + obs_of_lane(lane)] = (double)x;
     obs_warp_sums<NT>(d, local, step, tid, run, red, flag, sync, finish);
 }
 

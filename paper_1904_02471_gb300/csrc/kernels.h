@@ -41,7 +41,8 @@ inline cudaError_t launch_overlapped(const void* fn, int grid, int threads, void
 
 // Tile variants. CS: TX threads along x, RY rows per thread; the B
 // variants are the warp-specialised bulk-copy kernel (W columns x RB rows).
-// FD: TX x TY cells per tile, one cell per thread.
+// FD stages: 32 x TY nodes per tile, a block of march and preparing warps that
+// takes its SM whole; temporally blocked step: 32 x TY, a node or two per thread.
 enum CsTile { CS_T128x1 = 0, CS_T128x2, CS_T256x1, CS_T256x2, CS_T64x4, CS_B256x32, CS_B128x32, CS_T32x1, CS_NTILES };
 // FD_T32x1 (FP64 stages only) is picked by the default rule and the tuner, not
 // by configuration.

@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             // 2. per warp, one of: the moments of a row of each group (Eq.
             //    f_moments_discrete) with the observables of the state; the
             //    faces beyond the outermost lane, one (population, rows) per lane
-            double sum = 0.0;   // of observable `lane` over the warp's nodes
+            double sum = 0.0;   // of observable obs_of_lane(lane) over the warp's nodes
             constexpr int KX = Q1 * (Q1 - Q1 % 2);   // populations with faces along x
             constexpr int NE = (KX * H + 31) / 32;
             for (int task = aw; task < H + NE; task += NA) {
@@ -577,12 +577,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                                         v[3] = (pc == 0 ? P::get(jx, h) : P::get(jy, h)) / P::get(rho, h) * pxv * pyv;
                                     }
                                 }
-#pragma unroll
-                                for (int q = 0; q < NOBS; ++q) {
-#pragma unroll
-                                    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-                                }
-                                sum += (double)(lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3]);
+                                sum += (double)warp_obs_sums(v, lane);
                             }
                         }
                         if constexpr (!IMEX) e.set(rho, dr, jx, jy);
@@ -645,7 +640,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                 }
             }
             if (obs) {
-                if (lane < NOBS) red[aw * NOBS + lane] = sum;
+                if (lane < NOBS) red[aw * NOBS + obs_of_lane(lane)] = sum;
                 obs_warp_sums<NA * 32>(*cp, local, cp->step0 + j, atid, run, red, &s_last,
                                        [] { named_sync(1, NA * 32); }, g.finish_obs != 0);
             }
@@ -662,7 +657,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     for (unsigned n = 0;; ++n) {
         const int slot = n & 3;
         const int b = NB == 2 ? n & 1 : 0;
-            T* const buf = bufs + b * Ge::buf;
+        T* const buf = bufs + b * Ge::buf;
         const T* const mom = buf + (size_t)K * PL;
         const T* const edges = mom + Ge::n_mom;
         named_sync(2 + b, Ge::NT);

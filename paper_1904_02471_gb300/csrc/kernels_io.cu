@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(IO_THREADS) readout_kernel(const LatDesc* d, i
         acc[2] += jy;
         if (pc >= 0) acc[3] += (pc == 0 ? u : v) * d->probe_px[x] * d->probe_py[y];
     }
-    if (part) block_reduce_obs<double, IO_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
+    if (part) block_reduce_obs<IO_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
 }
 
 // Observables of the whole lattice (no readout): per node the moments in the
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(IO_THREADS) obs_snapshot_kernel(const LatDesc*
         acc[2] += (double)jy;
         if (pc >= 0) acc[3] += (double)((pc == 0 ? jx : jy) / (r0 + dr)) * d->probe_px[x] * d->probe_py[y];
     }
-    block_reduce_obs<double, IO_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
+    block_reduce_obs<IO_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
 }
 
 constexpr int FIN_THREADS = 256;

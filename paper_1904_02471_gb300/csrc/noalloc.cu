@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_partials_kernel(Noall
         acc[2] += (double)jy;
         if (a.comp >= 0) acc[3] += (double)((a.comp == 0 ? jx : jy) / ((T)a.rho0 + dr)) * a.px[x] * a.py[y];
     }
-    block_reduce_obs<double, NOALLOC_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
+    block_reduce_obs<NOALLOC_THREADS>(acc, part + (long long)blockIdx.x * NOBS, red);
 }
 
 __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_finalize_kernel(NoallocArgs a, const double* part,

@@ -98,11 +98,14 @@ void initial_fields(const lbm_request& q, std::vector<double>& rho, std::vector<
 
 // Estimated device time of one step of a run alone, for sharing the device
 // between runs: about 20 us of fixed cost per step (launch and tile latency
-// of a small lattice) plus a cost per node, from single-lattice rates on
-// GB300 (FP32: CS D2Q9 in place 74 GLUPS, FD 16-velocity 4.4 GLUPS, the FD
-// cost scaled by the number of velocities; FP64 on the narrow FP64 pipe; an
-// FD step with the IMEX scheme 1.1x, temporally blocked 3.0x the RK3 step,
-// as measured for FD 16-velocity 4096^2). Only the ratios between runs matter.
+// of a small lattice) plus a cost per node (FP32: CS D2Q9 in place 74 GLUPS, FD
+// 16-velocity 4.4 GLUPS, the FD cost scaled by the number of velocities; FP64
+// on the narrow FP64 pipe; an FD step with the IMEX scheme 1.1x, temporally
+// blocked 3.0x the RK3 step). Only the ratios between runs matter. The figures
+// are of the library's first kernels; the present ones run CS at 90 and FD
+// at 5.4 GLUPS, IMEX at 0.97 and the blocked step at 3.1 times the RK3 step, so
+// that the ratios hold to a third, and the round plans that follow from them
+// are part of the library's tests.
 double step_cost(const lbm_spec& s) {
     const double nodes = (double)s.nx * s.ny;
     const double k = (double)s.q_per_axis * s.q_per_axis;
@@ -126,7 +129,7 @@ void plan_round(const double* cost, const long long* left, size_t n, int chunk, 
 }
 
 // Runs whose estimated step (step_cost) takes this long or longer go to the
-// large-run lane: FD 16-velocity FP32 from 2048^2 (~1 ms), CS FP32 from
+// large-run lane: FD 16-velocity FP32 from 2048^2 (0.8 ms), CS FP32 from
 // about 6000^2.
 constexpr double kLargeStepCost = 0.5e-3;
 
