@@ -171,10 +171,6 @@ struct FdGeo {
     // per step of 2048^2, with eight 494.
     static constexpr int NA = Q1 == 4 || S == 2 ? (IMEX ? 8 : 4) : 7;
     static constexpr int NT = (NM + NA) * 32;
-    // registers per thread of the two kinds of warps (FP32, 16 velocities: the
-    // launch's registers are split between the warpgroups; 0: not split)
-    static constexpr bool SPLIT = Q1 == 4 && sizeof(T) == 4;
-    static constexpr int RM = SPLIT ? (IMEX ? 80 : 104) : 0, RA = SPLIT ? (IMEX ? 80 : 64) : 0;
     static constexpr size_t n_mom = (size_t)5 * TY * FD_TX;
     static constexpr size_t n_edge = ((size_t)K * TY + 3) / 4 * 4;
     static constexpr size_t buf = (size_t)K * PL + n_mom + n_edge;   // values of a tile buffer
@@ -367,7 +363,6 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
     const bool node_in = IMEX || stage != 1;
 
     if (warp >= NM) {
-        if constexpr (Ge::RA > 0) set_regs_dec<Ge::RA>();
         // ---- preparing warps: look up the block's items, copy their tiles,
         //      form their moments and outer faces, one item ahead of the march
         const int aw = warp - NM, atid = tid - NM * 32;
@@ -481,7 +476,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     const int x = e < nl ? e - 3 : xr + e - nl;
                     const T* s = U0 + ((unsigned)wrap_near(y0 - 3 + r, ny) * (unsigned)pitch + (unsigned)wrap_near(x, nx));
                     T* t = buf + r * HXP + (x - x0 + 4);
-#pragma unroll 4
+#pragma unroll 1
                     for (int k = 0; k < K; ++k, s += plane, t += PL)
                         if (LBM_BC_NODE(cp, K, s - U0)) cp_async_small<sizeof(T)>(t, s);
                 }
@@ -557,7 +552,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                             // float values, as with a node per thread), the rest
                             // in double
                             const int pc = cp->probe_comp, y = y0 + r;
-#pragma unroll
+#pragma unroll 1
                             for (int h = 0; h < N; ++h) {
                                 const int x = x0 + c0 + h;
                                 T v[NOBS] = {T(0), T(0), T(0), T(0)};
@@ -649,7 +644,6 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
         return;
     }
 
-    if constexpr (Ge::RM > 0) set_regs_inc<Ge::RM>();
     // ---- march warps
     // stage weights: f^(s) = f^n + cb ((u - f^n) + dt L(u)), i.e. the Shu-Osher
     // combinations 3/4 f^n + 1/4 (u + dt L(u)) and 1/3 f^n + 2/3 (u + dt L(u))
@@ -840,18 +834,16 @@ int fd_tile_ty(int v) {
     return 0;
 }
 
-// A kernel variant: its entry, block size, dynamic shared memory and, where
-// the warpgroups split the launch's registers, the registers of their shares.
+// A kernel variant: its entry, block size and dynamic shared memory.
 struct FdVariant {
     const void* fn = nullptr;
     int threads = 0;
     size_t bytes = 0;
-    int regs = 0;
 };
 template <typename T, int Q1, int TY, bool IMEX>
 static FdVariant fd_variant_of() {
     using Ge = FdGeo<T, Q1, TY, IMEX>;
-    return FdVariant{(const void*)fd_stage_kernel<T, Q1, TY, IMEX>, Ge::NT, Ge::bytes, 32 * (Ge::NM * Ge::RM + Ge::NA * Ge::RA)};
+    return FdVariant{(const void*)fd_stage_kernel<T, Q1, TY, IMEX>, Ge::NT, Ge::bytes};
 }
 template <typename T, int Q1, bool IMEX>
 static FdVariant fd_variant_q(int tile) {
@@ -899,11 +891,7 @@ static cudaError_t fd_prepare(int precision, int tile, int q1) {
     }
     for (int scheme : {LBM_TS_RK3, LBM_TS_IMEX}) {
         const FdVariant v = fd_variant(precision, tile, q1, scheme);
-        cudaFuncAttributes a;
-        if (!v.fn || v.bytes > (size_t)optin || cudaFuncGetAttributes(&a, v.fn) != cudaSuccess ||
-            // the shares must not exceed the registers the block is launched
-            // with (a warpgroup would wait for the rest for ever)
-            v.regs > (a.numRegs + 7) / 8 * 8 * v.threads ||
+        if (!v.fn || v.bytes > (size_t)optin ||
             cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.bytes) != cudaSuccess) {
             cudaGetLastError();
             st = 2;

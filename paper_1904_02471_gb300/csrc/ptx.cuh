@@ -118,15 +118,4 @@ __device__ __forceinline__ void after_previous_launch() {
     allow_next_launch();
 }
 
-// Change the registers per thread of the calling warpgroup (four aligned
-// warps, all of them executing it) within those the block was launched with.
-template <int N>
-__device__ __forceinline__ void set_regs_inc() {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N>
-__device__ __forceinline__ void set_regs_dec() {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
-}
-
 }  // namespace lbm
