@@ -493,6 +493,10 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
             auto at = [&](int k, int r, int c) {
                 return buf + k * PL + (r + 3) * HXP + c + 4;
             };
+            // FP32: the map below sums the moments of Y, kept for the tile's own nodes (a
+            // pass of their own took 1 to 3% of a step); FP64, whose pipe is the
+            // bound, sums them for the tile's nodes only (map: 2 to 7% slower)
+            constexpr bool SUM_Y = IMEX && sizeof(T) == 4;
             if constexpr (IMEX) {
                 // the implicit BGK part of the stage in closed form, at every
                 // staged node: the stage value Y solves Y = u + dt g C(Y), C(Y) =
@@ -510,23 +514,25 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     Equil<T> e;
                     e.set(P::add(P::sp(r0), dr), dr, jx, jy);
                     const EquilAll<T, Q1> ea(e);
-                    // map and sum the moments of Y (summed in a pass of their own,
-                    // they took 3 to 6% of a step); kept for the tile's own nodes
-                    set_moments<T, Q1>(
-                        [&](int k) {
-                            const V geq = P::mulc(ea.over_w(k), (T)w_of<Q1>(k));
-                            T* u = at(k, r, c);
-                            const V y = P::mul(P::fma(vlam, geq, ldv_again(u)), vil);
-                            stv(u, y);
-                            return y;
-                        },
-                        dr, jx, jy);
-                    if (r >= 0 && r < TY && c >= 0 && c < TX) {
-                        e.set(P::add(P::sp(r0), dr), dr, jx, jy);
-                        T* m = mo + 2 * (r * TX + c);
-                        stv2(m, e.px, e.py);
-                        stv2(m + 2 * TY * TX, e.jx, e.jy);
-                        stv(mo + 4 * TY * TX + r * TX + c, e.e0);
+                    auto map = [&](int k) {
+                        const V geq = P::mulc(ea.over_w(k), (T)w_of<Q1>(k));
+                        T* u = at(k, r, c);
+                        const V y = P::mul(P::fma(vlam, geq, ldv_again(u)), vil);
+                        stv(u, y);
+                        return y;
+                    };
+                    if constexpr (SUM_Y) {
+                        set_moments<T, Q1>(map, dr, jx, jy);
+                        if (r >= 0 && r < TY && c >= 0 && c < TX) {
+                            e.set(P::add(P::sp(r0), dr), dr, jx, jy);
+                            T* m = mo + 2 * (r * TX + c);
+                            stv2(m, e.px, e.py);
+                            stv2(m + 2 * TY * TX, e.jx, e.jy);
+                            stv(mo + 4 * TY * TX + r * TX + c, e.e0);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < K; ++k) map(k);
                     }
                 }
                 named_sync(1, NA * 32);
@@ -543,7 +549,7 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                     const int r = task + grp * H;   // tile row
                     T* m = mo + 2 * (r * TX + c0);
                     Equil<T> e;
-                    if (!IMEX || obs) {
+                    if (!SUM_Y || obs) {
                         V dr, jx, jy;
                         set_moments<T, Q1>([&](int k) { return ldv(at(k, r, c0)); }, dr, jx, jy);
                         const V rho = P::add(P::sp(r0), dr);
@@ -575,9 +581,9 @@ __global__ void __launch_bounds__(FdGeo<T, Q1, TY, IMEX>::NT, 1) fd_stage_kernel
                                 sum += (double)warp_obs_sums(v, lane);
                             }
                         }
-                        if constexpr (!IMEX) e.set(rho, dr, jx, jy);
+                        if constexpr (!SUM_Y) e.set(rho, dr, jx, jy);
                     }
-                    if constexpr (IMEX) {
+                    if constexpr (SUM_Y) {
                         ldv2(m, e.px, e.py);
                         ldv2(m + 2 * TY * TX, e.jx, e.jy);
                         e.e0 = ldv(mo + 4 * TY * TX + r * TX + c0);
