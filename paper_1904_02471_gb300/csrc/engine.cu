@@ -143,8 +143,9 @@ void Engine::invalidate_graph() {
 // step, one block per work item (tile; the hardware scheduler balances the
 // tiles; the tuner picked this for every workload measured, e.g. CS D2Q9 8192^2
 // in place 90 GLUPS against 72 with one block set per SM); FD stages, one block
-// per SM (a block prepares its next tile while it works on one: 1.06 ms per
-// stage of FD 16-velocity 4096^2 against 1.7 ms with one block per tile). One
+// per SM (a block prepares its next tile while it works on one: 0.98 ms per
+// stage of FD 16-velocity 4096^2; 1.06 against 1.7 ms with one block per tile
+// when this was chosen). One
 // block set per SM for a server's engine,
 // whose lattices change under a captured graph (the blocks then loop over
 // the items), or grid_mult_ block sets, so that each block covers fewer items

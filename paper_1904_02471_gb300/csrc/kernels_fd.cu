@@ -295,8 +295,8 @@ constexpr double IMEX_GAMMA = 0.29289321881345247560;
 // per stage of FD 16-velocity 4096^2 FP32 however the tile was cut). Here the
 // preparing warps' work overlaps the march, which never waits for memory: f^n
 // is loaded a march ahead, the rest is in shared memory. Stages of that lattice:
-// 1.19 / 1.13 / 1.13 -> 0.96 / 1.00 / 1.03 ms; FP64 256^2: 275 -> 200 us (fewer
-// operations per face and node, one reciprocal instead of a division).
+// 1.19 / 1.13 / 1.13 -> 0.98 / 0.98 / 0.99 ms; FP64 256^2: 275 -> 198 us per stage
+// (fewer operations per face and node, one reciprocal instead of a division).
 // Named barriers hand the buffers over: waiting warps take no issue slots
 // (polling an mbarrier took 10% of them).
 //

@@ -103,7 +103,7 @@ void initial_fields(const lbm_request& q, std::vector<double>& rho, std::vector<
 // on the narrow FP64 pipe; an FD step with the IMEX scheme 1.1x, temporally
 // blocked 3.0x the RK3 step). Only the ratios between runs matter. The figures
 // are of the library's first kernels; the present ones run CS at 90 and FD
-// at 5.4 GLUPS, IMEX at 0.97 and the blocked step at 3.1 times the RK3 step, so
+// at 5.7 GLUPS, IMEX at 1.0 and the blocked step at 3.2 times the RK3 step, so
 // that the ratios hold to a third, and the round plans that follow from them
 // are part of the library's tests.
 double step_cost(const lbm_spec& s) {
