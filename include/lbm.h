@@ -350,8 +350,11 @@ int lbm_batch_step_profiled(lbm_batch* b, int64_t n, double* ms, int cap, double
  * tile variant 0 .. lbm_n_tiles(model)-1 and grid size (blocks loop over the
  * group's work items; 0 picks the default: for CS and the temporally blocked
  * FD step one block per work item, i.e. per tile of every lattice of the
- * group, for FD stages at most one block per SM). Every variant computes bit-identical
- * results; only speed differs. lbm_config does the same for a context. */
+ * group, for FD stages at most one block per SM). Every variant computes
+ * bit-identical populations; only speed differs, and the last bits of recorded
+ * observables, whose sums are formed per tile and block (a fixed order for
+ * a tile and grid). The default tile of a CS group follows its recording
+ * (lbm_record). lbm_config does the same for a context. */
 int lbm_batch_config(lbm_batch* b, int group, int tile, int grid);
 int lbm_config(lbm_ctx* ctx, int tile, int grid);
 int lbm_n_tiles(int model);
@@ -363,7 +366,8 @@ int64_t lbm_kernel_launches(const lbm_ctx* ctx);
 
 /* Autotuner: times the candidate tile shapes and grid sizes of every group
  * of the batch on its current state (state is saved and restored) and keeps
- * the fastest; results are cached per (model, q, precision, size class).
+ * the fastest; the tile and the kind of grid are cached for sets of the same
+ * model, q, precision, scheme, sizes, storage and recording interval.
  * trial_steps > 0 steps per candidate. Writes a one-line summary into
  * report (may be NULL) of report_len bytes. */
 int lbm_batch_tune(lbm_batch* b, int trial_steps, char* report, size_t report_len);
